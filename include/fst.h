@@ -67,7 +67,7 @@ typedef enum {
  * fst_plan -- precomputation of Section 1.3 (last paragraph) and Section 4.1.
  * Computes, on the GPU in FP64, the Slepian basis vectors of the eigen-window
  * around K (bisection on Slepian's commuting tridiagonal matrix, split by parity,
- * then inverse iteration), their eigenvalues lambda_l = s_l^T B s_l (FP64 FFT
+ * then a forward recurrence), their eigenvalues lambda_l = s_l^T B s_l (FP64 FFT
  * convolution), the transition set T = {l : |1[l<K] - lambda_l| > eps}, D, the
  * real sinc spectrum DFT_M(c) (FP64, stored FP32 and FP64) and the twiddle tables.
  *   out     receives the new plan (owned by the library; free with fst_destroy).

@@ -36,7 +36,7 @@ template <typename T> struct DevEx {
 };
 
 struct NoState {
-  c2<double> v[1];
+  int top;
 };
 struct DevExPlan {
   using State = NoState;
@@ -130,13 +130,42 @@ template <typename T> __global__ void __launch_bounds__(1024) k_passC(const Conv
 // plan kernels
 // ---------------------------------------------------------------------------
 
-__global__ void k_bisect_ms_many(const TargetDesc *td, const double *dcat, const double *e2cat, double *theta,
-                                 int *flag) {
-  __shared__ BisectShared sh;
-  DevExPlan ex;
-  const TargetDesc q = td[blockIdx.x];
-  bisect_body(ex, dcat + q.mat_off, e2cat + q.mat_off, q.n, q.target, q.glo, q.ghi, q.pivmin, q.tol, theta + blockIdx.x,
-              flag, &sh);
+// One round of multisection: warp w of target t narrows the target's interval with the counts of
+// the previous round (every warp of a target does so by itself; its first one keeps the result
+// for the next round), then counts at its 32 points.  iv: [2][nt][lo, hi], cnt: [2][nt][32 warps],
+// the halves alternate with the round.  The last call (eval = 0) only narrows.  Blocks of four
+// warps: one on each sub-core's FP64 unit.
+constexpr int BISECT_THREADS = 128;
+__global__ void __launch_bounds__(BISECT_THREADS) k_bisect_round(const TargetDesc *td, int nt, int warps, int round, int eval,
+                                                     const double *dcat, const double *e2cat, double *iv, int *cnt,
+                                                     double *theta, int *flag) {
+  const int gw = blockIdx.x * (BISECT_THREADS / 32) + (threadIdx.x >> 5);
+  const int t = gw / warps, w = gw % warps, lane = threadIdx.x & 31, np = 32 * warps;
+  if (t >= nt) return;
+  const TargetDesc q = td[t];
+  double lo = q.glo, hi = q.ghi;
+  if (round > 0) {
+    const double *ivp = iv + ((size_t)((round - 1) & 1) * nt + t) * 2;
+    const int *cp = cnt + ((size_t)((round - 1) & 1) * nt + t) * np;
+    int k = 0;
+    for (int i = lane; i < np; i += 32) k += cp[i] <= q.target;
+    k = __reduce_add_sync(0xffffffffu, k);
+    lo = ivp[0];
+    hi = ivp[1];
+    bisect_narrow(&lo, &hi, k, np);
+  }
+  if (w == 0 && lane == 0) {
+    double *ivn = iv + ((size_t)(round & 1) * nt + t) * 2;
+    ivn[0] = lo;
+    ivn[1] = hi;
+    if (!eval) {
+      theta[t] = 0.5 * (lo + hi);
+      if (!bisect_converged(lo, hi, q.tol)) *flag = 1;
+    }
+  }
+  if (eval)
+    cnt[((size_t)(round & 1) * nt + t) * np + 32 * w + lane] =
+        sturm_count(dcat + q.mat_off, e2cat + q.mat_off, q.n, bisect_point(lo, hi, 32 * w + lane, np), q.pivmin);
 }
 
 __global__ void k_bisect_many(const TargetDesc *td, int nt, const double *dcat, const double *e2cat, double *theta,
@@ -146,20 +175,22 @@ __global__ void k_bisect_many(const TargetDesc *td, int nt, const double *dcat, 
   const TargetDesc q = td[t];
   bisect1_body(dcat + q.mat_off, e2cat + q.mat_off, q.n, q.target, q.glo, q.ghi, q.pivmin, q.tol, theta + t, flag);
 }
-__global__ void k_invit_many(const TargetDesc *td, int nt, const double *dcat, const double *ecat,
-                             const double *theta, double *x, double *fd, double *fdl, double *fdu, double *fdu2,
-                             uint8_t *piv) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
-  if (t >= nt) return;
+// `lanes` targets per one-warp block
+__global__ void __launch_bounds__(32) k_fwdvec_many(const TargetDesc *td, int nt, int lanes, const double *dcat,
+                                                    const double *ecat, const double *rcat, const double *theta,
+                                                    double *z, double *w, int *ex, double *delta) {
+  const int t = blockIdx.x * lanes + threadIdx.x;
+  if ((int)threadIdx.x >= lanes || t >= nt) return;
   const TargetDesc q = td[t];
-  invit_body(dcat + q.mat_off, ecat + q.mat_off, q.n, theta[t], q.tol, 3, 0, 1, x + q.x_off, fd + q.x_off,
-             fdl + q.x_off, fdu + q.x_off, fdu2 + q.x_off, piv + q.x_off);
+  fwdvec_body(dcat + q.mat_off, ecat + q.mat_off, rcat + q.mat_off, q.n, theta[t], z + q.x_off, w + q.x_off,
+              ex + q.x_off / PLAN_B, delta + t);
 }
-__global__ void k_finalize_many(const TargetDesc *td, const double *x) {
+__global__ void k_finalize_many(const TargetDesc *td, const double *z, const double *w, const int *bex,
+                                const double *delta) {
   __shared__ double sh[2 * 256];
   DevExPlan ex;
   const TargetDesc q = td[blockIdx.x];
-  finalize_body(ex, x + q.x_off, q.n, 1, 0, q.parity, q.N, q.S, sh);
+  finalize_body(ex, z + q.x_off, w + q.x_off, bex + q.x_off / PLAN_B, delta[blockIdx.x], q.n, q.parity, q.N, q.S, sh);
 }
 
 __global__ void k_dot(const double *a, const double *b, int64_t N, double *out) {
@@ -987,11 +1018,14 @@ struct DevRunner : Runner {
   }
   fst_status passC(const ConvArgs<double> &a, const Layout &L) override { return passC_t(a, L); }
 
-  fst_status bisect_ms_many(const TargetDesc *td, int nt, const double *dcat, const double *e2cat, double *theta,
-                            int *flag) override {
+  fst_status bisect_ms_many(const TargetDesc *td, int nt, int warps, int rounds, const double *dcat,
+                            const double *e2cat, double *iv, int *cnt, double *theta, int *flag) override {
     if (nt <= 0) return FST_OK;
-    PROF_S(s, "k_bisect_ms_many", nt, (k_bisect_ms_many<<<nt, BISECT_THREADS, 0, s>>>(td, dcat, e2cat, theta, flag)));
-    LAUNCHED("k_bisect_ms_many");
+    for (int r = 0; r <= rounds; ++r) {
+      const int last = r == rounds;
+      PROF_S(s, "k_bisect_round", nt, (k_bisect_round<<<(nt * warps * 32 + BISECT_THREADS - 1) / BISECT_THREADS, BISECT_THREADS, 0, s>>>(td, nt, warps, r, !last, dcat, e2cat, iv, cnt, theta, flag)));
+      LAUNCHED("k_bisect_round");
+    }
     return FST_OK;
   }
   fst_status bisect_many(const TargetDesc *td, int nt, const double *dcat, const double *e2cat, double *theta,
@@ -1001,14 +1035,18 @@ struct DevRunner : Runner {
     LAUNCHED("k_bisect_many");
     return FST_OK;
   }
-  fst_status invit_many(const TargetDesc *td, int nt, const double *dcat, const double *ecat, const double *theta,
-                        double *x, double *fd, double *fdl, double *fdu, double *fdu2, uint8_t *piv) override {
-    PROF_S(s, "k_invit_many", nt, (k_invit_many<<<(nt + 63) / 64, 64, 0, s>>>(td, nt, dcat, ecat, theta, x, fd, fdl, fdu, fdu2, piv)));
-    LAUNCHED("k_invit_many");
+  fst_status fwdvec_many(const TargetDesc *td, int nt, const double *dcat, const double *ecat, const double *rcat,
+                         const double *theta, double *z, double *w, int *ex, double *delta) override {
+    // spread over the SMs: a warp's FP64 instruction takes its SM's pipe equally long with any
+    // number of active lanes
+    const int lanes = std::max(1, std::min(32, (nt + sms - 1) / sms));
+    PROF_S(s, "k_fwdvec_many", nt, (k_fwdvec_many<<<(nt + lanes - 1) / lanes, 32, 0, s>>>(td, nt, lanes, dcat, ecat, rcat, theta, z, w, ex, delta)));
+    LAUNCHED("k_fwdvec_many");
     return FST_OK;
   }
-  fst_status finalize_many(const TargetDesc *td, int nt, const double *x) override {
-    PROF_S(s, "k_finalize_many", nt, (k_finalize_many<<<nt, 256, 0, s>>>(td, x)));
+  fst_status finalize_many(const TargetDesc *td, int nt, const double *z, const double *w, const int *ex,
+                           const double *delta) override {
+    PROF_S(s, "k_finalize_many", nt, (k_finalize_many<<<nt, 256, 0, s>>>(td, z, w, ex, delta)));
     LAUNCHED("k_finalize_many");
     return FST_OK;
   }

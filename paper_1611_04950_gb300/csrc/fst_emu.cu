@@ -24,7 +24,7 @@ template <typename S> struct HostEx {
   }
 };
 struct NoStateH {
-  c2<double> v[1];
+  int top;
 };
 
 struct EmuRunner : Runner {
@@ -131,14 +131,20 @@ struct EmuRunner : Runner {
   fst_status passC(const ConvArgs<float> &a, const Layout &L) override { return passC_t(a, L); }
   fst_status passC(const ConvArgs<double> &a, const Layout &L) override { return passC_t(a, L); }
 
-  fst_status bisect_ms_many(const TargetDesc *td, int nt, const double *dcat, const double *e2cat, double *theta,
-                            int *flag) override {
+  fst_status bisect_ms_many(const TargetDesc *td, int nt, int warps, int rounds, const double *dcat,
+                            const double *e2cat, double *, int *, double *theta, int *flag) override {
+    const int np = 32 * warps;
     for (int t = 0; t < nt; ++t) {
       const TargetDesc &q = td[t];
-      BisectShared sh;
-      HostEx<NoStateH> ex(BISECT_THREADS);
-      bisect_body(ex, dcat + q.mat_off, e2cat + q.mat_off, q.n, q.target, q.glo, q.ghi, q.pivmin, q.tol, theta + t, flag,
-                  &sh);
+      double lo = q.glo, hi = q.ghi;
+      for (int r = 0; r < rounds; ++r) {
+        int k = 0;
+        for (int i = 0; i < np; ++i)
+          k += sturm_count(dcat + q.mat_off, e2cat + q.mat_off, q.n, bisect_point(lo, hi, i, np), q.pivmin) <= q.target;
+        bisect_narrow(&lo, &hi, k, np);
+      }
+      theta[t] = 0.5 * (lo + hi);
+      if (!bisect_converged(lo, hi, q.tol)) *flag = 1;
     }
     return FST_OK;
   }
@@ -150,21 +156,22 @@ struct EmuRunner : Runner {
     }
     return FST_OK;
   }
-  fst_status invit_many(const TargetDesc *td, int nt, const double *dcat, const double *ecat, const double *theta,
-                        double *x, double *fd, double *fdl, double *fdu, double *fdu2, uint8_t *piv) override {
+  fst_status fwdvec_many(const TargetDesc *td, int nt, const double *dcat, const double *ecat, const double *rcat,
+                         const double *theta, double *z, double *w, int *ex, double *delta) override {
     for (int t = 0; t < nt; ++t) {
       const TargetDesc &q = td[t];
-      invit_body(dcat + q.mat_off, ecat + q.mat_off, q.n, theta[t], q.tol, 3, 0, 1, x + q.x_off, fd + q.x_off,
-                 fdl + q.x_off, fdu + q.x_off, fdu2 + q.x_off, piv + q.x_off);
+      fwdvec_body(dcat + q.mat_off, ecat + q.mat_off, rcat + q.mat_off, q.n, theta[t], z + q.x_off, w + q.x_off,
+                  ex + q.x_off / PLAN_B, delta + t);
     }
     return FST_OK;
   }
-  fst_status finalize_many(const TargetDesc *td, int nt, const double *x) override {
+  fst_status finalize_many(const TargetDesc *td, int nt, const double *z, const double *w, const int *bex,
+                           const double *delta) override {
     std::vector<double> sh(2 * 256);
     for (int t = 0; t < nt; ++t) {
       const TargetDesc &q = td[t];
       HostEx<NoStateH> ex(256);
-      finalize_body(ex, x + q.x_off, q.n, 1, 0, q.parity, q.N, q.S, sh.data());
+      finalize_body(ex, z + q.x_off, w + q.x_off, bex + q.x_off / PLAN_B, delta[t], q.n, q.parity, q.N, q.S, sh.data());
     }
     return FST_OK;
   }

@@ -539,13 +539,13 @@ struct PendingWin {
 };
 
 // The window vectors of a group of plans: both parities of every plan's window as one batch of
-// independent targets (bisection, inverse iteration one thread per target, expansion).
+// independent targets (bisection, forward recurrence one thread per target, expansion).
 static fst_status batched_window_vectors(std::vector<PendingWin *> &grp) {
   if (grp.empty()) return FST_OK;
   Runner *R0 = grp[0]->p->R;
   Scoped sc(R0);
   // concatenated reduced matrices and one descriptor per target
-  std::vector<double> dcat, ecat, e2cat;
+  std::vector<double> dcat, ecat, e2cat, rcat;
   std::vector<TargetDesc> td;
   for (PendingWin *pw : grp) {
     fst_plan_t p = pw->p;
@@ -566,6 +566,10 @@ static fst_status batched_window_vectors(std::vector<PendingWin *> &grp) {
       dcat.insert(dcat.end(), red.d.begin(), red.d.end());
       ecat.insert(ecat.end(), red.e.begin(), red.e.end());
       e2cat.insert(e2cat.end(), red.e2.begin(), red.e2.end());
+      for (int i = 0; i < red.n; ++i) rcat.push_back(i + 1 < red.n ? 1.0 / red.e[i + 1] : 1.0);
+      // the next matrix begins on a whole block of PLAN_B entries
+      for (std::vector<double> *v : {&dcat, &ecat, &e2cat, &rcat})
+        v->resize((v->size() + PLAN_B - 1) / PLAN_B * PLAN_B, 0.0);
       for (int64_t l = pw->lo; l <= pw->hi; ++l) {
         if ((l & 1) != parity) continue;
         TargetDesc q{};
@@ -579,59 +583,74 @@ static fst_status batched_window_vectors(std::vector<PendingWin *> &grp) {
         q.glo = glo - widen;
         q.ghi = ghi + widen;
         q.pivmin = pivmin;
-        // pivot lift of the inverse iteration and absolute floor of the bisection's stopping
-        // test; > 0 also for a zero matrix (N = 1)
+        // absolute floor of the bisection's stopping test; > 0 also for a zero matrix (N = 1)
         q.tol = 2.220446049250313e-16 * tnorm + pivmin;
         td.push_back(q);
       }
     }
   }
   const int nt = (int)td.size();
-  double *dd, *de, *de2, *theta;
+  // the kernels load up to two blocks past a matrix's end
+  for (std::vector<double> *v : {&dcat, &ecat, &e2cat, &rcat}) v->resize(v->size() + 2 * PLAN_B, 0.0);
+  double *dd, *de, *de2, *dr, *theta;
   int *flag;
   TargetDesc *dtd;
   TRY(sc.alloc(&dd, dcat.size()));
   TRY(sc.alloc(&de, ecat.size()));
   TRY(sc.alloc(&de2, e2cat.size()));
+  TRY(sc.alloc(&dr, rcat.size()));
   TRY(sc.alloc(&theta, nt));
   TRY(sc.alloc(&flag, 1));
   TRY(sc.alloc(&dtd, nt));
   TRY(R0->h2d(dd, dcat.data(), dcat.size() * sizeof(double)));
   TRY(R0->h2d(de, ecat.data(), ecat.size() * sizeof(double)));
   TRY(R0->h2d(de2, e2cat.data(), e2cat.size() * sizeof(double)));
+  TRY(R0->h2d(dr, rcat.data(), rcat.size() * sizeof(double)));
   TRY(R0->zero(flag, sizeof(int)));
   TRY(R0->h2d(dtd, td.data(), td.size() * sizeof(TargetDesc)));
-  // few targets: multisection, one block each (fewer rounds; the GPU has room for the extra
-  // Sturm counts); many: plain bisection, one thread each (less arithmetic in all)
-  if (nt <= BISECT_MS_MAX_TARGETS) TRY(R0->bisect_ms_many(dtd, nt, dd, de2, theta, flag));
-  else TRY(R0->bisect_many(dtd, nt, dd, de2, theta, flag));
+  // few targets: multisection (fewer rounds; the GPU has room for the extra Sturm counts), as
+  // many warps per target as give every SM four, which its FP64 units run side by side; many:
+  // plain bisection, one thread each (less arithmetic in all).  N = 65536, 44 targets: 13 warps
+  // each, 6 rounds, 27.7 ms (one block of 64 points per target and 9 rounds: 79.9 ms)
+  if (nt <= BISECT_MS_MAX_TARGETS) {
+    const int warps = std::max(1, std::min(BISECT_WARPS_MAX, (R0->device() ? 4 : 1) * R0->sm_count() / std::max(nt, 1)));
+    double bits = 1.0;
+    for (const TargetDesc &q : td) bits = std::max(bits, log2((q.ghi - q.glo) / q.tol));
+    const int rounds = (int)ceil(bits / log2(32.0 * warps + 1.0));
+    double *iv;
+    int *cnt;
+    TRY(sc.alloc(&iv, (size_t)4 * nt));
+    TRY(sc.alloc(&cnt, (size_t)64 * warps * nt));
+    TRY(R0->bisect_ms_many(dtd, nt, warps, rounds, dd, de2, iv, cnt, theta, flag));
+  } else {
+    TRY(R0->bisect_many(dtd, nt, dd, de2, theta, flag));
+  }
   int hflag = 0;
   TRY(R0->d2h(&hflag, flag, sizeof(int)));
   if (hflag) return fail(FST_ENOCONVERGE, "bisection did not converge");
-  // inverse iteration and expansion in groups bounded by the factor storage
-  const int64_t budget = 192LL << 20;   // elements per factor array (41 bytes each in all)
+  // vectors and expansion in groups bounded by their storage; a target's arrays begin on a
+  // whole block of PLAN_B entries
+  const int64_t budget = 192LL << 20;   // elements of z and of w
   for (int t0 = 0; t0 < nt;) {
     int t1 = t0;
     int64_t tot = 0;
     while (t1 < nt && (tot + td[t1].n <= budget || t1 == t0)) {
       td[t1].x_off = tot;
-      tot += td[t1].n;
+      tot += (td[t1].n + PLAN_B - 1) / PLAN_B * PLAN_B;
       ++t1;
     }
     Scoped g(R0);
-    double *x, *fd, *fdl, *fdu, *fdu2;
-    uint8_t *piv;
+    double *z, *w, *delta;
+    int *ex;
     TargetDesc *gtd;
-    TRY(g.alloc(&x, tot));
-    TRY(g.alloc(&fd, tot));
-    TRY(g.alloc(&fdl, tot));
-    TRY(g.alloc(&fdu, tot));
-    TRY(g.alloc(&fdu2, tot));
-    TRY(g.alloc(&piv, tot));
+    TRY(g.alloc(&z, tot));
+    TRY(g.alloc(&w, tot));
+    TRY(g.alloc(&ex, tot / PLAN_B));
+    TRY(g.alloc(&delta, t1 - t0));
     TRY(g.alloc(&gtd, t1 - t0));
     TRY(R0->h2d(gtd, td.data() + t0, (size_t)(t1 - t0) * sizeof(TargetDesc)));
-    TRY(R0->invit_many(gtd, t1 - t0, dd, de, theta + t0, x, fd, fdl, fdu, fdu2, piv));
-    TRY(R0->finalize_many(gtd, t1 - t0, x));
+    TRY(R0->fwdvec_many(gtd, t1 - t0, dd, de, dr, theta + t0, z, w, ex, delta));
+    TRY(R0->finalize_many(gtd, t1 - t0, z, w, ex, delta));
     TRY(R0->sync());
     t0 = t1;
   }
@@ -1513,8 +1532,8 @@ fst_status fst_adi_shifts(int64_t N, int r, double *out) {
 
 // ===========================================================================
 // Many plans at once (ragged batches): the eigen stage of every plan's window
-// runs as one batch of independent targets (bisection and inverse iteration one
-// thread per target), the rest per plan.
+// runs as one batch of independent targets (bisection and eigenvectors one thread
+// per target), the rest per plan.
 // ===========================================================================
 namespace fst {
 

@@ -108,15 +108,18 @@ struct Runner {
 
   // plan kernels (all pointers in runner memory)
   // batched eigen-targets of one or many plans (descriptors and data in runner memory):
-  // multisection (a block of BISECT_THREADS per target) or plain bisection (a thread per target)
-  virtual fst_status bisect_ms_many(const TargetDesc *td, int nt, const double *dcat, const double *e2cat,
-                                    double *theta, int *flag) = 0;
+  // multisection (`warps` warps of 32 points per target and round; iv: 4 nt doubles, cnt:
+  // 64 warps nt ints of scratch) or plain bisection (a thread per target)
+  virtual fst_status bisect_ms_many(const TargetDesc *td, int nt, int warps, int rounds, const double *dcat,
+                                    const double *e2cat, double *iv, int *cnt, double *theta, int *flag) = 0;
   virtual fst_status bisect_many(const TargetDesc *td, int nt, const double *dcat, const double *e2cat,
                                  double *theta, int *flag) = 0;
-  virtual fst_status invit_many(const TargetDesc *td, int nt, const double *dcat, const double *ecat,
-                                const double *theta, double *x, double *fd, double *fdl, double *fdu, double *fdu2,
-                                uint8_t *piv) = 0;
-  virtual fst_status finalize_many(const TargetDesc *td, int nt, const double *x) = 0;
+  // reduced eigenvectors z, their derivatives w, block exponents and eigenvalue corrections
+  virtual fst_status fwdvec_many(const TargetDesc *td, int nt, const double *dcat, const double *ecat,
+                                 const double *rcat, const double *theta, double *z, double *w, int *ex,
+                                 double *delta) = 0;
+  virtual fst_status finalize_many(const TargetDesc *td, int nt, const double *z, const double *w, const int *ex,
+                                   const double *delta) = 0;
   virtual fst_status dot(const double *a, const double *b, int64_t N, int nvec, double *out) = 0;
   virtual fst_status sinc_embed(double *c, int64_t N, int64_t M, double W) = 0;
   virtual fst_status spec_store(const double2 *X, const Layout &L64, const Layout &L32, int64_t M, double scale,

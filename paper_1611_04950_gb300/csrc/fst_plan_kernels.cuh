@@ -11,9 +11,9 @@
 //   N = 2m+1:  symmetric: leading (m+1) x (m+1) block with the coupling between
 //              m-1 and m multiplied by sqrt(2) (the centre sample is sqrt(2) u_m);
 //              antisymmetric: leading m x m block (the centre sample is 0).
-// Bodies here: multisection bisection on Sturm counts, inverse iteration with
-// partially pivoted tridiagonal LU, and the expansion of a reduced vector to the
-// unit-norm, sign-fixed full vector.
+// Bodies here: multisection bisection on Sturm counts, the eigenvector by the forward
+// three-term recurrence with a first-order correction of the eigenvalue, and the expansion
+// of a reduced vector to the unit-norm, sign-fixed full vector.
 #pragma once
 #include <math.h>
 #include <stdint.h>
@@ -22,9 +22,9 @@
 
 namespace fst {
 
-constexpr int BISECT_THREADS = 64;
 constexpr int BISECT_MS_MAX_TARGETS = 512;   // batches up to this many targets use multisection
-constexpr int BISECT_MAX_ROUNDS = 24;
+constexpr int BISECT_WARPS_MAX = 16;         // warps (32 points each) per target and round
+constexpr int PLAN_B = 8;                    // steps of a serial recurrence whose inputs are loaded ahead
 
 // biased exponent field of a double (0 for zeros and subnormals)
 FST_HD int dexp_field(double v) {
@@ -37,86 +37,148 @@ FST_HD int dexp_field(double v) {
 #endif
 }
 
+// 2^k as a double, -1022 <= k <= 1023
+FST_HD double dpow2(int k) {
+  const uint64_t u = (uint64_t)(k + 1023) << 52;
+#ifdef __CUDA_ARCH__
+  return __longlong_as_double((long long)u);
+#else
+  double v;
+  memcpy(&v, &u, 8);
+  return v;
+#endif
+}
+
+// The FP64 unit of this part, measured: an FP64 instruction holds its warp for 64 clocks whatever
+// its active lanes and dependences, up to four warps per SM (one per sub-core) run side by side at
+// 76, and more only queue.  So the serial recurrences below count FP64 instructions: signs, zeros
+// and exponents are tested on the integer pipe, and rare FP64 work sits behind a branch that a
+// warp takes as one (any lane needs it), which the compiler cannot turn into selects.
+FST_HD int dneg(double v) {
+#ifdef __CUDA_ARCH__
+  return (int)((unsigned)__double2hiint(v) >> 31);
+#else
+  return v < 0.0;
+#endif
+}
+FST_HD bool warp_any(bool v) {
+#ifdef __CUDA_ARCH__
+  return __any_sync(__activemask(), v);
+#else
+  return v;
+#endif
+}
+FST_HD bool dzero(double v) {
+#ifdef __CUDA_ARCH__
+  return ((__double2hiint(v) & 0x7fffffff) | __double2loint(v)) == 0;
+#else
+  return v == 0.0;
+#endif
+}
+
+// PLAN_B consecutive entries (the concatenated matrices begin on multiples of PLAN_B entries and
+// are followed by 2 PLAN_B spare ones, so blocks are aligned and may be loaded past the end)
+FST_HD void load_block(const double *a, double *v) {
+#pragma unroll
+  for (int k = 0; k < PLAN_B; k += 2) {
+#ifdef __CUDA_ARCH__
+    const double2 q = __ldg(reinterpret_cast<const double2 *>(a + k));
+    v[k] = q.x;
+    v[k + 1] = q.y;
+#else
+    v[k] = a[k];
+    v[k + 1] = a[k + 1];
+#endif
+  }
+}
+
 // Number of eigenvalues of the reduced matrix smaller than x: the sign changes of the Sturm
 // sequence of leading principal minors p_i = det(T_i - x I), p_i = (d_i - x) p_{i-1} -
-// e_i^2 p_{i-2} (p_{-1} = 1), which equal the negative pivots q_i = p_i / p_{i-1} of
+// e_i^2 p_{i-2} (p_{-1} = 1, e_0 = 0), which equal the negative pivots q_i = p_i / p_{i-1} of
 // T - x I = L D L^T.  The recurrence needs no division (the serial chain is one FMA per step);
-// every 4 steps the pair (p_i, p_{i-1}) is rescaled by an exact power of two when both are
-// beyond 2^(+-400) (a step grows them by at most about 2^87 for N <= 2^23), and an exact zero
-// p_i is replaced by -pivmin p_{i-1} (the pivot -pivmin of the LDL^T form).
+// every PLAN_B steps the pair (p_i, p_{i-1}) is brought back to exponent 0 by an exact power of
+// two when it has left 2^(+-128) (a step grows it by at most about 2^87 for N <= 2^23, so a block
+// stays below 2^824), and an exact zero p_i is replaced by -pivmin p_{i-1} (the pivot -pivmin of the LDL^T form).
+// Bound: the FP64 unit.  A step is 3 FP64 instructions (product, difference, FMA); zeros are
+// looked for once per block, whose steps are then taken again one by one; the inputs of the next
+// block are loaded while the current one is processed.  Measured at N = 65536 (32768 steps, four
+// warps per SM): a test and branch in every step 6.1 ms a round, one per block 4.6 ms.
 FST_HD int sturm_count(const double *d, const double *e2, int n, double x, double pivmin) {
-  double pm = 1.0, p = ldg(d) - x;
-  if (p == 0.0) p = -pivmin;
-  int c = (p < 0.0);
-  for (int i = 1; i < n; ++i) {
-    const double t = ldg(e2 + i) * pm;
-    double pn = fma(ldg(d + i) - x, p, -t);
-    if (pn == 0.0) pn = -pivmin * p;
-    c += ((pn < 0.0) != (p < 0.0));
-    pm = p;
-    p = pn;
-    if ((i & 3) == 0) {
-      const int ex = dexp_field(p), exm = dexp_field(pm);
-      const int mx = ex > exm ? ex : exm;
-      if (mx > 1023 + 400) {
-        p *= 0x1p-512;
-        pm *= 0x1p-512;
-      } else if (mx < 1023 - 400) {
-        p *= 0x1p512;
-        pm *= 0x1p512;
+  constexpr int B = PLAN_B;
+  double pm = 0.0, p = 1.0;
+  int neg = 0, c = 0;
+  double E[B], D[B], En[B], Dn[B];
+  // steps [k0, k1) of the block held in D, E, with the zero test in each
+  auto slow = [&](int k1) {
+    for (int k = 0; k < k1; ++k) {
+      double pn = fma(D[k] - x, p, -(E[k] * pm));
+      if (dzero(pn)) pn = -pivmin * p;
+      const int ng = dneg(pn);
+      c += ng ^ neg;
+      neg = ng;
+      pm = p;
+      p = pn;
+    }
+  };
+  load_block(e2, E);
+  load_block(d, D);
+  int i0 = 0;
+  for (; i0 + B <= n; i0 += B) {
+    load_block(e2 + i0 + B, En);
+    load_block(d + i0 + B, Dn);
+    const double p0 = p, pm0 = pm;
+    const int neg0 = neg, c0 = c;
+    bool zero = false;
+#pragma unroll
+    for (int k = 0; k < B; ++k) {
+      const double pn = fma(D[k] - x, p, -(E[k] * pm));
+      zero = zero || dzero(pn);
+      const int ng = dneg(pn);
+      c += ng ^ neg;
+      neg = ng;
+      pm = p;
+      p = pn;
+    }
+    const int ex = dexp_field(p), exm = dexp_field(pm), mx = ex > exm ? ex : exm;
+    if (warp_any(zero || mx > 1023 + 128 || mx < 1023 - 128)) {
+      if (zero) {
+        p = p0;
+        pm = pm0;
+        neg = neg0;
+        c = c0;
+        slow(B);
       }
+      const int a = dexp_field(p), b = dexp_field(pm), m = a > b ? a : b;
+      const double f = (m > 1023 + 128 || m < 1023 - 128) ? dpow2(1023 - (m > 1 ? m : 1)) : 1.0;
+      p *= f;
+      pm *= f;
+    }
+#pragma unroll
+    for (int k = 0; k < B; ++k) {
+      E[k] = En[k];
+      D[k] = Dn[k];
     }
   }
+  slow(n - i0);
   return c;
 }
 
-struct BisectShared {
-  double lo, hi;
-  int done;
-  int cnt[BISECT_THREADS];
-};
-
-// Block computes the eigenvalue of ascending index `target` of the reduced matrix:
-// each round evaluates the Sturm count at 64 interior points of [lo, hi] and keeps
-// the sub-interval that holds it (6 bits per round), until the interval is within 4 ulp
-// of its ends plus abstol (about eps ||T||: an eigenvalue near 0, e.g. every transition
-// eigenvalue at W = 1/4 where the diagonal vanishes, needs no more for the inverse
-// iteration).  flag != 0 on non-convergence.
-template <typename Ex>
-FST_HD void bisect_body(Ex &ex, const double *d, const double *e2, int n, int target, double glo, double ghi,
-                        double pivmin, double abstol, double *out, int *flag, BisectShared *sh) {
-  using St = typename Ex::State;
-  ex.phase([&](int tid, St &) {
-    if (tid == 0) { sh->lo = glo; sh->hi = ghi; sh->done = 0; }
-  });
-  for (int round = 0; round < BISECT_MAX_ROUNDS; ++round) {
-    ex.phase([&](int tid, St &) {
-      const double lo = sh->lo, hi = sh->hi;
-      const double x = lo + (hi - lo) * (double)(tid + 1) / (double)(BISECT_THREADS + 1);
-      sh->cnt[tid] = sturm_count(d, e2, n, x, pivmin);
-    });
-    ex.phase([&](int tid, St &) {
-      if (tid == 0) {
-        const double lo = sh->lo, hi = sh->hi;
-        int t = 0;
-        while (t < BISECT_THREADS && sh->cnt[t] <= target) ++t;
-        // count(x_t) > target >= count(x_{t-1}): eigenvalue in [x_{t-1}, x_t]
-        const double nlo = (t == 0) ? lo : lo + (hi - lo) * (double)t / (double)(BISECT_THREADS + 1);
-        const double nhi = (t == BISECT_THREADS) ? hi : lo + (hi - lo) * (double)(t + 1) / (double)(BISECT_THREADS + 1);
-        sh->lo = nlo;
-        sh->hi = nhi;
-        const double tol = 4.0 * 2.220446049250313e-16 * fmax(fabs(nlo), fabs(nhi)) + abstol;
-        if (nhi - nlo <= tol || (nlo == lo && nhi == hi)) sh->done = 1;
-      }
-    });
-    if (sh->done) break;
-  }
-  ex.phase([&](int tid, St &) {
-    if (tid == 0) {
-      *out = 0.5 * (sh->lo + sh->hi);
-      if (!sh->done) *flag = 1;
-    }
-  });
+// One round of multisection: the Sturm counts of np interior points of a target's interval
+// [lo, hi] (any number of warps, on any SMs) leave the sub-interval that holds the eigenvalue.
+//   point k < np of [lo, hi]: lo + (hi - lo) (k + 1) / (np + 1)
+//   k = number of points whose count is <= target: the eigenvalue lies in [x_{k-1}, x_k]
+// The interval ends within 4 ulp of its ends plus abstol (about eps ||T||: an eigenvalue near 0,
+// e.g. every transition eigenvalue at W = 1/4 where the diagonal vanishes, needs no more).
+FST_HD double bisect_point(double lo, double hi, int k, int np) {
+  return lo + (hi - lo) * (double)(k + 1) / (double)(np + 1);
+}
+FST_HD void bisect_narrow(double *lo, double *hi, int k, int np) {
+  const double a = *lo, b = *hi;
+  if (k > 0) *lo = bisect_point(a, b, k - 1, np);
+  if (k < np) *hi = bisect_point(a, b, k, np);
+}
+FST_HD bool bisect_converged(double lo, double hi, double abstol) {
+  return hi - lo <= 4.0 * 2.220446049250313e-16 * fmax(fabs(lo), fabs(hi)) + abstol;
 }
 
 // Plain bisection for one target (one thread), used when many plans are built at
@@ -141,195 +203,120 @@ FST_HD void bisect1_body(const double *d, const double *e2, int n, int target, d
 // Descriptor of one eigen-target of a batch of plans (fst_plan_many).
 struct TargetDesc {
   int64_t mat_off;   // reduced matrix: d, e, e2 at [mat_off, mat_off + n) of the concatenations
-  int64_t x_off;     // this target's vector and factor arrays at [x_off, x_off + n)
+  int64_t x_off;     // this target's vector and derivative at [x_off, x_off + n), exponents at x_off / 8
   double *S;         // output: the full unit-norm Slepian vector (length N)
   int64_t N;
   int n, target, parity, pad_;
   double glo, ghi, pivmin, tol;
 };
 
-// Inverse iteration for one eigenvalue sigma of the reduced matrix (diag d,
-// coupling e[i] between i-1 and i): LU with partial pivoting of T - sigma I (the
-// classical tridiagonal elimination; row interchanges create a second
-// superdiagonal), zero pivots lifted to tol, then `iters` solves with the same
-// factors, each followed by scaling to max-norm 1.  Vector t of nt: element i at
-// [i * nt + t] in x and in the factor arrays.  fd holds the reciprocals of the
-// (lifted) U diagonal, so the back substitution multiplies.
-//
-// Each phase is a serial chain over i.  The entries a step updates travel to the next
-// step in registers (cd, cu: U diagonal and super-diagonal at i; cur: x[i]; x1, x2:
-// x[i+1], x[i+2]), and the inputs of the next INVIT_B steps are loaded while the current
-// ones are processed (the loads never touch an entry the current block writes), so the
-// chain waits on arithmetic, not on memory.
-constexpr int INVIT_B = 8;
-FST_HD void invit_body(const double *d, const double *e, int n, double sigma, double tol, int iters, int t, int nt,
-                       double *x, double *fd, double *fdl, double *fdu, double *fdu2, uint8_t *piv) {
-#define AT(a, i) a[(int64_t)(i) * nt + t]
-  constexpr int B = INVIT_B;
-  auto lift = [&](double p) { return (fabs(p) < tol) ? ((p < 0.0) ? -tol : tol) : p; };
-  // ---- factor: steps i = 0 .. n-2 read e[i+1], d[i+1], e[i+2]
-  {
-    double cd = ldg(d) - sigma;
-    double cu = (n > 1) ? ldg(e + 1) : 0.0;
-    double E[B + 1], D[B];
-    auto load = [&](int i0, double *Ev, double *Dv) {
-#pragma unroll
-      for (int k = 0; k <= B; ++k) Ev[k] = (i0 + 1 + k < n) ? ldg(e + i0 + 1 + k) : 0.0;
-#pragma unroll
-      for (int k = 0; k < B; ++k) Dv[k] = (i0 + 1 + k < n) ? ldg(d + i0 + 1 + k) : 0.0;
+// Eigenvector of the reduced matrix (diag d, coupling e[i] between i-1 and i, r[i] = 1 / e[i+1])
+// for the eigenvalue sigma, by its own rows from the edge to the centre:
+//   z_0 = 1,  z_{i+1} = -((d_i - sigma) z_i + e_i z_{i-1}) / e_{i+1}.
+// Row x from the centre (s = x^2, A = N^2/4) reads sigma = C s + (A - s) cos(phi), C = cos 2 pi W,
+// so cos(phi) = (sigma - C s) / (A - s) is monotonic in s: every Slepian vector oscillates around
+// the centre and has at most one region without oscillation, at the edge, where the recurrence
+// follows the growing solution.  It is therefore stable for every index, each row is met to its
+// own rounding, and only the last row is left with a residual, which is due to the rounding of
+// sigma.  That is removed to first order with the derivative w = dz / d sigma,
+//   (T - sigma) w = z on the same rows,  delta = -(last row of z) / (its derivative),
+// and the vector is z + delta w (delta is a fraction of an ulp of ||T||).
+// z and w are scaled by 2^256 at block ends (PLAN_B entries) when they leave 2^(+-128); ex holds
+// each block's exponent.  A step grows them by at most about N/2 (at the edge), a block by less
+// than 2^176, so one factor is enough and squares stay finite.
+// Bound: a serial chain of n steps of 7 FP64 instructions of 64 clocks each; inputs are loaded
+// PLAN_B steps ahead.  Measured at N = 65536 (44 targets of n = 32768): 7.8 ms; the inverse
+// iteration with a partially pivoted LU that this replaced took 73.9 ms and left vectors
+// orthogonal to 1e-11 where these reach 1e-13 (N = 86679, W = 0.0185).
+FST_HD void fwdvec_body(const double *d, const double *e, const double *r, int n, double sigma, double *z, double *w,
+                        int *ex, double *delta) {
+  constexpr int B = PLAN_B;
+  double zc = 1.0, zm = 0.0, wc = 0.0, wm = 0.0, rz = 0.0, rw = 0.0;
+  int sh = 0;
+  double D[B], E[B], R[B], Dn[B], En[B], Rn[B];
+  load_block(d, D);
+  load_block(e, E);
+  load_block(r, R);
+  for (int i0 = 0; i0 < n; i0 += B) {
+    load_block(d + i0 + B, Dn);
+    load_block(e + i0 + B, En);
+    load_block(r + i0 + B, Rn);
+    ex[i0 / B] = sh;
+    auto step = [&](int k) {
+      z[i0 + k] = zc;
+      w[i0 + k] = wc;
+      const double a = D[k] - sigma;
+      rz = fma(a, zc, E[k] * zm);
+      rw = fma(a, wc, fma(E[k], wm, -zc));
+      zm = zc;
+      wm = wc;
+      zc = -rz * R[k];
+      wc = -rw * R[k];
     };
-    load(0, E, D);
-    for (int i0 = 0; i0 + 1 < n; i0 += B) {
-      double En[B + 1], Dn[B];
-      load(i0 + B, En, Dn);
+    if (i0 + B <= n) {
 #pragma unroll
-      for (int k = 0; k < B; ++k) {
-        const int i = i0 + k;
-        if (i + 1 < n) {
-          const double li = E[k], nd = D[k] - sigma, nu = (i + 2 < n) ? E[k + 1] : 0.0;
-          if (fabs(cd) >= fabs(li)) {
-            const double f = (cd != 0.0) ? li / cd : 0.0;
-            AT(fdl, i) = f;
-            AT(fd, i) = 1.0 / lift(cd);
-            AT(fdu, i) = cu;
-            AT(fdu2, i) = 0.0;
-            AT(piv, i) = 0;
-            cd = nd - f * cu;
-            cu = nu;
-          } else {
-            const double f = cd / li;
-            AT(fdl, i) = f;
-            AT(fd, i) = 1.0 / lift(li);
-            AT(fdu, i) = nd;
-            AT(fdu2, i) = nu;
-            AT(piv, i) = 1;
-            cd = cu - f * nd;
-            cu = -f * nu;
-          }
-        }
-      }
+      for (int k = 0; k < B; ++k) step(k);
+    } else {
 #pragma unroll
-      for (int k = 0; k <= B; ++k) E[k] = En[k];
-#pragma unroll
-      for (int k = 0; k < B; ++k) D[k] = Dn[k];
+      for (int k = 0; k < B; ++k)
+        if (i0 + k < n) step(k);
     }
-    AT(fd, n - 1) = 1.0 / lift(cd);
-    AT(fdu, n - 1) = 0.0;
-    AT(fdl, n - 1) = 0.0;
-    AT(fdu2, n - 1) = 0.0;
-    AT(piv, n - 1) = 0;
-  }
-  // start vector: deterministic, no structure shared with any eigenvector
-  for (int i = 0; i < n; ++i) {
-    const double g = (double)i * 0.6180339887498949;
-    AT(x, i) = 0.5 + (g - floor(g));
-  }
-  for (int it = 0; it < iters; ++it) {
-    // ---- L solve with the row interchanges: step i reads x[i+1] (not yet written), fdl[i], piv[i]
-    {
-      double cur = AT(x, 0);
-      double X[B], L[B];
-      unsigned PV;
-      auto load = [&](int i0, double *Xv, double *Lv, unsigned &pv) {
-        pv = 0u;
-#pragma unroll
-        for (int k = 0; k < B; ++k) {
-          const bool ok = i0 + k + 1 < n;
-          Xv[k] = ok ? AT(x, i0 + k + 1) : 0.0;
-          Lv[k] = ok ? AT(fdl, i0 + k) : 0.0;
-          pv |= (ok && AT(piv, i0 + k)) ? (1u << k) : 0u;
-        }
-      };
-      load(0, X, L, PV);
-      for (int i0 = 0; i0 + 1 < n; i0 += B) {
-        double Xn[B], Ln[B];
-        unsigned PVn;
-        load(i0 + B, Xn, Ln, PVn);
-#pragma unroll
-        for (int k = 0; k < B; ++k) {
-          const int i = i0 + k;
-          if (i + 1 < n) {
-            if (((PV >> k) & 1u) == 0u) {
-              AT(x, i) = cur;
-              cur = X[k] - L[k] * cur;
-            } else {
-              AT(x, i) = X[k];
-              cur = cur - L[k] * X[k];
-            }
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < B; ++k) {
-          X[k] = Xn[k];
-          L[k] = Ln[k];
-        }
-        PV = PVn;
-      }
-      AT(x, n - 1) = cur;
+    const int ea = dexp_field(zc), eb = dexp_field(zm), mx = ea > eb ? ea : eb;
+    if (warp_any(mx > 1023 + 128 || mx < 1023 - 128)) {
+      const double f = mx > 1023 + 128 ? 0x1p-256 : (mx < 1023 - 128 ? 0x1p256 : 1.0);
+      zc *= f;
+      zm *= f;
+      wc *= f;
+      wm *= f;
+      sh += mx > 1023 + 128 ? 256 : (mx < 1023 - 128 ? -256 : 0);
     }
-    // ---- U solve (descending), max-norm: step i reads x[i], fdu[i], fdu2[i], fd[i]
-    double mx = 0.0;
-    {
-      double x1 = 0.0, x2 = 0.0;
-      double X[B], U1[B], U2[B], R[B];
-      auto load = [&](int i1, double *Xv, double *U1v, double *U2v, double *Rv) {
 #pragma unroll
-        for (int k = 0; k < B; ++k) {
-          const int i = i1 - k;
-          const bool ok = i >= 0;
-          Xv[k] = ok ? AT(x, i) : 0.0;
-          U1v[k] = ok ? AT(fdu, i) : 0.0;
-          U2v[k] = ok ? AT(fdu2, i) : 0.0;
-          Rv[k] = ok ? AT(fd, i) : 0.0;
-        }
-      };
-      load(n - 1, X, U1, U2, R);
-      for (int i1 = n - 1; i1 >= 0; i1 -= B) {
-        double Xn[B], U1n[B], U2n[B], Rn[B];
-        load(i1 - B, Xn, U1n, U2n, Rn);
-#pragma unroll
-        for (int k = 0; k < B; ++k) {
-          const int i = i1 - k;
-          if (i >= 0) {
-            double v = X[k];
-            if (i + 1 < n) v -= U1[k] * x1;
-            if (i + 2 < n) v -= U2[k] * x2;
-            v *= R[k];
-            AT(x, i) = v;
-            mx = fmax(mx, fabs(v));
-            x2 = x1;
-            x1 = v;
-          }
-        }
-#pragma unroll
-        for (int k = 0; k < B; ++k) {
-          X[k] = Xn[k];
-          U1[k] = U1n[k];
-          U2[k] = U2n[k];
-          R[k] = Rn[k];
-        }
-      }
+    for (int k = 0; k < B; ++k) {
+      D[k] = Dn[k];
+      E[k] = En[k];
+      R[k] = Rn[k];
     }
-    const double s = (mx > 0.0) ? 1.0 / mx : 1.0;
-    for (int i = 0; i < n; ++i) AT(x, i) = AT(x, i) * s;
   }
-#undef AT
+  const double dl = -rz / rw;   // the last row's residual over its derivative
+  *delta = (dl - dl == 0.0) ? dl : 0.0;
 }
 
-// Expansion of reduced vector t (interleaved x[i * nt + t], size n, parity p) to the
+// Expansion of a reduced vector (z + delta w with block exponents ex, size n, parity p) to the
 // full unit-norm Slepian vector s (length N, contiguous) with the sign convention:
 // symmetric vectors have positive sum, antisymmetric ones positive
-// sum((N-1-2i) s[i]).  Block reduction in a fixed order.  sh: 2 * nthr doubles.
+// sum((N-1-2i) s[i]).  Block reductions in a fixed order.  sh: 2 * nthr doubles.
 template <typename Ex>
-FST_HD void finalize_body(Ex &ex, const double *x, int n, int nt, int t, int parity, int64_t N, double *s, double *sh) {
+FST_HD void finalize_body(Ex &ex, const double *z, const double *w, const int *bex, double delta, int n, int parity,
+                          int64_t N, double *s, double *sh) {
   using St = typename Ex::State;
   const int nthr = ex.nthr;
   const bool odd = (N & 1) != 0;
   const int64_t m = N / 2;  // full index m is the centre when N is odd
+  // entry i over 2^(largest block exponent)
+  auto entry = [&](int64_t i, int top) {
+    const int k = bex[i / PLAN_B] - top;
+    return (k < -1792) ? 0.0 : fma(delta, w[i], z[i]) * ldexp(1.0, k < -1000 ? -1000 : k) * (k < -1000 ? ldexp(1.0, k + 1000) : 1.0);
+  };
   ex.phase([&](int tid, St &) {
+    int top = -2147483647;
+    for (int i = tid; i < (n + PLAN_B - 1) / PLAN_B; i += nthr) top = bex[i] > top ? bex[i] : top;
+    sh[tid] = (double)top;
+  });
+  ex.phase([&](int tid, St &) {
+    if (tid == 0) {
+      double top = sh[0];
+      for (int k = 1; k < nthr; ++k) top = fmax(top, sh[k]);
+      sh[nthr] = top;
+    }
+  });
+  // (the sums below reuse sh: the exponent travels in the last slot until it is read)
+  ex.phase([&](int tid, St &st) {
+    st.top = (int)sh[nthr];
+  });
+  ex.phase([&](int tid, St &st) {
     double nrm = 0.0, ref = 0.0;
     for (int i = tid; i < n; i += nthr) {
-      const double u = x[(int64_t)i * nt + t];
+      const double u = entry(i, st.top);
       nrm += u * u;
       if (parity == 0) ref += (odd && i == m) ? 0.7071067811865476 * u : u;  // centre counts once, times sqrt(2)/2
       else ref += (double)(N - 1 - 2 * (int64_t)i) * u;
@@ -346,20 +333,19 @@ FST_HD void finalize_body(Ex &ex, const double *x, int n, int nt, int t, int par
       sh[0] = scale;
     }
   });
-  ex.phase([&](int tid, St &) {
+  ex.phase([&](int tid, St &st) {
     const double scale = sh[0];
     const double sgn = (parity == 0) ? 1.0 : -1.0;
-    for (int64_t i = tid; i < N; i += nthr) {
-      double v;
+    for (int64_t i = tid; i < n; i += nthr) {
+      const double v = entry(i, st.top) * scale;
       if (odd && i == m) {
-        v = (parity == 0) ? 1.4142135623730951 * x[(int64_t)m * nt + t] * scale : 0.0;
-      } else if (i < m || (odd && i < m)) {
-        v = x[i * nt + t] * scale;
+        s[i] = 1.4142135623730951 * v;
       } else {
-        v = sgn * x[(N - 1 - i) * nt + t] * scale;
+        s[i] = v;
+        s[N - 1 - i] = sgn * v;
       }
-      s[i] = v;
     }
+    if (odd && parity == 1 && tid == 0) s[m] = 0.0;
   });
 }
 
