@@ -18,6 +18,7 @@
 #include "../../include/fst_testing.h"
 #include "fst_fast.cuh"
 #include "fst_big.cuh"
+#include "fst_fast64.cuh"
 #define FST_TC_KERNELS
 #include "fst_tc.cuh"
 
@@ -112,7 +113,8 @@ template <typename T> __global__ void k_reduce(const ConvArgs<T> a) {
   reduce_body<T>(a, (int64_t)blockIdx.x, threadIdx.x, blockDim.x);
 }
 
-template <typename T> __global__ void __launch_bounds__(1024) k_passB(const ConvArgs<T> a) {
+// (FP64 rows have at most 8192 points)
+template <typename T> __global__ void __launch_bounds__(sizeof(T) == 8 ? 512 : 1024) k_passB(const ConvArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem[];
   c2<T> *buf = reinterpret_cast<c2<T> *>(smem);
   DevEx<T> ex;
@@ -878,6 +880,56 @@ struct DevRunner : Runner {
     return FST_OK;
   }
   fst_status passB(const ConvArgs<double> &a, const Layout &L) override { return passB_t(a, L); }
+  // Tile sizes: a block of 512 values (four warps, one per sub-core) once that makes two blocks per
+  // SM; otherwise as small as 128 values (one warp), so that a single short signal spreads over
+  // more SMs.  One pair of N = 4096: 39.7 us; with 512-value tiles 41.5.
+  fst_status f64_passes(const ConvArgs<double> &a, int spec_log2P, int pass) override {
+    TRY(set_attrs());
+    F64Args f{a, spec_log2P, 0, 0};
+    const int P = 1 << a.log2P, Q = 1 << a.log2Q;
+    const int64_t vals = a.npairs << a.log2M;
+    int tile = vals >= 512LL * 2 * sms ? 512 : 128;
+    if (pass == 1 && a.log2Q >= 11 && spec_log2P == a.log2P) {
+      dim3 grid((unsigned)P, (unsigned)a.npairs);
+      PROF("k_passB<f64>", a.npairs, (k_passB<double><<<grid, Q / 16, padded_size(Q) * 16, cur>>>(a)));
+      LAUNCHED("k_passB");
+      return FST_OK;
+    }
+    auto lg = [](int v) { int l = 0; while ((2 << l) <= v) ++l; return l; };
+    if (pass == 1) {
+      f.log2RT = lg(std::max(1, std::min(P, tile / Q)));
+      const int64_t blocks = (a.npairs * P) >> f.log2RT;
+      PROF("k_f64B", a.npairs, (k_f64B<<<(unsigned)blocks, (Q << f.log2RT) / 4, ((size_t)Q << f.log2RT) * 16, cur>>>(f)));
+      LAUNCHED("k_f64B");
+      return FST_OK;
+    }
+    f.log2NB = lg(std::min(Q, tile / P));
+    const int64_t blocks = a.npairs * (Q >> f.log2NB);
+    const size_t smem = ((size_t)P << f.log2NB) * 16;
+    if (pass == 0) PROF("k_f64A", a.npairs, (k_f64A<<<(unsigned)blocks, (P << f.log2NB) / 4, smem, cur>>>(f)));
+    else PROF("k_f64C", a.npairs, (k_f64C<<<(unsigned)blocks, (P << f.log2NB) / 4, smem, cur>>>(f)));
+    LAUNCHED("k_f64A/C");
+    return FST_OK;
+  }
+  fst_status f64_corr(const ConvArgs<double> &a, const unsigned char *cpar, int64_t rows, int chunk, double *part,
+                      double *acoef) override {
+    const int64_t H = (a.N + 1) / 2;
+    const int nchunk = (int)((H + chunk - 1) / chunk);
+    const int64_t rg = (rows + F64_RG - 1) / F64_RG;
+    if (rg > 65535 || (rows * a.r + 7) / 8 >= (1LL << 31)) return fail(FST_EINVAL, "batch too large for the FP64 correction");
+    PROF("k_f64_corr", rows, (k_f64_corr<<<dim3((unsigned)nchunk, (unsigned)rg), 256, 0, cur>>>(a, cpar, chunk, rows, part)));
+    LAUNCHED("k_f64_corr");
+    PROF("k_f64_reduce", rows, (k_f64_reduce<<<(unsigned)((rows * a.r + 7) / 8), 256, 0, cur>>>(a, nchunk, rows, part, acoef)));
+    LAUNCHED("k_f64_reduce");
+    return FST_OK;
+  }
+  fst_status f64_z(const ConvArgs<double> &a, const unsigned char *cpar, int64_t rows, const double *acoef) override {
+    const int64_t H = (a.N + 1) / 2;
+    dim3 grid((unsigned)((H + F64_ZN - 1) / F64_ZN), (unsigned)((rows + F64_ZR - 1) / F64_ZR));
+    PROF("k_f64_z", rows, (k_f64_z<<<grid, F64_ZN * F64_ZR, 0, cur>>>(a, cpar, rows, acoef)));
+    LAUNCHED("k_f64_z");
+    return FST_OK;
+  }
   fst_status corr_c(const ConvArgs<float> &a) override {
     FastArgs f{a, a.ST_hl};
     dim3 grid((unsigned)((a.N + CORR_BLOCK - 1) / CORR_BLOCK), (unsigned)((a.npairs + FAST_G - 1) / FAST_G));

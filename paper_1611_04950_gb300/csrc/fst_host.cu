@@ -280,6 +280,78 @@ static fst_status ensure_ws(fst_plan_t p, size_t bytes) {
   return FST_OK;
 }
 
+// FP64 four-step path of fst_fast64.cuh: M = 2^10 .. 2^18.  The split is P = 32, or for batches whose
+// rows fill the GPU that of the plan's FP64 layout (rows of at least 2048 points, the faster row
+// kernel).  The plan's spectrum keeps its own order (natural up to M = 2^13).
+struct F64Plan {
+  bool on = false;
+  int log2P = 0, log2Q = 0, chunk = 0, nchunk = 0;   // chunk: folded samples per partial of S_T^T y
+  int64_t group = 0;                                 // pairs per launch group
+  size_t inter_b = 0, part_b = 0, acoef_b = 0;
+};
+static F64Plan f64_plan(fst_plan_t p, int64_t npairs, bool cplx, int64_t batch, bool full) {
+  F64Plan f;
+  // (rows beyond 4 * 65535 do not fit the grid of the S_T a pass: the generic kernels take those)
+  if (!p->R->device() || p->log2M < 10 || p->log2M > 18 || !p->cpar || (cplx ? 2 : 1) * batch > 4 * 65535) return f;
+  f.on = true;
+  f.log2P = 5;
+  if (!p->lay64.small && (npairs << p->lay64.log2P) >= 2 * p->R->sm_count()) f.log2P = p->lay64.log2P;
+  f.log2Q = p->log2M - f.log2P;
+  f.group = std::max<int64_t>(1, std::min<int64_t>(npairs, chunk_bytes_target() >> (p->log2M + 4)));
+  f.inter_b = ((size_t)f.group << (p->log2M + 4));
+  if (full && p->r > 0) {
+    // partials over chunks of at least one 32-sample tile; about four blocks per SM in all
+    const int64_t rows = cplx ? 2 * batch : batch, H = (p->N + 1) / 2, rg = (rows + 7) / 8;
+    const int64_t want = std::max<int64_t>(1, 4 * (int64_t)p->R->sm_count() / rg);
+    f.chunk = (int)(((H + want - 1) / want + 31) / 32 * 32);
+    f.nchunk = (int)((H + f.chunk - 1) / f.chunk);
+    f.part_b = (size_t)f.nchunk * rows * p->rpad * sizeof(double);
+    f.acoef_b = (size_t)rows * p->rpad * sizeof(double);
+  }
+  return f;
+}
+static fst_status run_f64(fst_plan_t p, const F64Plan &f, ConvArgs<double> a, int64_t npairs, char *ws) {
+  Runner *R = p->R;
+  const int lanes = R->lanes();
+  a.log2M = p->log2M;
+  a.log2P = f.log2P;
+  a.log2Q = f.log2Q;
+  a.Pnz = (int)((a.N + (1LL << f.log2Q) - 1) >> f.log2Q);
+  const int64_t rows = a.cplx ? 2 * a.batch : a.batch;
+  double *part = (double *)(ws + (size_t)lanes * f.inter_b), *acoef = (double *)((char *)part + f.part_b);
+  const bool corr = f.nchunk > 0;
+  if (corr) {
+    // reads every signal before pass C writes any output (y == out works)
+    R->use_side();
+    TRY(R->f64_corr(a, p->cpar, rows, f.chunk, part, acoef));
+    R->side_done();
+  }
+  bool waited[2] = {!corr, !corr};
+  int64_t g = 0;
+  for (int64_t p0 = 0; p0 < npairs; p0 += f.group, ++g) {
+    const int lane = (int)(g % lanes);
+    R->use_lane(lane);
+    a.inter = (double2 *)(ws + (size_t)lane * f.inter_b);
+    a.pair0 = p0;
+    a.npairs = std::min<int64_t>(f.group, npairs - p0);
+    for (int pass = 0; pass < 3; ++pass) {
+      if (pass == 2 && !waited[lane]) {
+        R->wait_side();
+        waited[lane] = true;
+      }
+      TRY(R->f64_passes(a, p->lay64.small ? 0 : p->lay64.log2P, pass));
+    }
+  }
+  R->use_lane(0);
+  if (corr) {
+    R->lanes_join_first();
+    R->wait_side();
+    TRY(R->f64_z(a, p->cpar, rows, acoef));
+  }
+  return FST_OK;
+}
+static fst_status run_f64(fst_plan_t, const F64Plan &, ConvArgs<float>, int64_t, char *) { return FST_EUNSUPPORTED; }
+
 template <typename T>
 static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64_t ld, bool cplx, bool full,
                           const T *spec, const T *ST, const T *D, const Layout &L0, void *ext_ws,
@@ -309,7 +381,7 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
   const int64_t npairs = cplx ? batch : (batch + 1) / 2;
   const bool dbl = sizeof(T) == 8;
   const bool sep = (L0.split_corr || (p->STt && !L0.small && !dbl)) && full && p->r > 0;
-  const size_t extra = sep ? split_corr_bytes(p->N, npairs, (int)p->rpad) : 0;
+  const size_t sep_b = sep ? split_corr_bytes(p->N, npairs, (int)p->rpad) : 0;
   if (!ext_ws) {
     Runner *R = p->R;
     // launch groups no larger than the call needs (small batches, ragged signals)
@@ -322,12 +394,15 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
       TRY(ensure_ws(p, ws_need(Lp, false, (int)p->rpad, false)));
       return run_conv<T>(R, Lp, a, npairs, p->ws);
     }
-    const size_t slot = ws_need(Lc, dbl, (int)p->rpad, false);
+    const F64Plan f64 = dbl ? f64_plan(p, npairs, cplx, batch, full) : F64Plan();
+    const size_t slot = f64.on ? f64.inter_b : ws_need(Lc, dbl, (int)p->rpad, false);
+    const size_t extra = f64.on ? f64.part_b + f64.acoef_b : sep_b;
+    auto run = [&]() { return f64.on ? run_f64(p, f64, a, npairs, (char *)p->ws) : run_conv<T>(R, Lc, a, npairs, p->ws); };
     const bool graphs = R->device() && graphs_enabled() && !profiling_enabled() && !tc_stall_pending() &&
                         !R->user_stream_capturing();
     if (!graphs) {
       TRY(ensure_ws(p, slot + extra));
-      return run_conv<T>(R, Lc, a, npairs, p->ws);
+      return run();
     }
     // whole apply as one cached CUDA graph (two overlapping lanes of launch groups)
     for (auto &e : p->graphs)
@@ -335,10 +410,8 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
           e.dtype == (int)(cplx ? 1 : 0) + (dbl ? 2 : 0) && e.full == full)
         return R->graph_launch(e.exec, e.nodes);
     TRY(ensure_ws(p, 2 * slot + 256 + extra));
-    if (!R->graph_begin()) {
-      return run_conv<T>(R, Lc, a, npairs, p->ws);
-    }
-    fst_status st = run_conv<T>(R, Lc, a, npairs, p->ws);
+    if (!R->graph_begin()) return run();
+    fst_status st = run();
     const std::string first_err = st != FST_OK ? std::string(g_err) : std::string();
     void *exec = nullptr;
     long long nodes = 0;
@@ -362,11 +435,11 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
     int64_t ch = L.chunk;
     while (ch > L.G) {
       L.chunk = ch;
-      if (ws_need(L, dbl, (int)p->rpad, false) + extra <= ext_bytes) break;
+      if (ws_need(L, dbl, (int)p->rpad, false) + sep_b <= ext_bytes) break;
       ch = std::max<int64_t>(L.G, ((ch / 2) / L.G) * L.G);
     }
     L.chunk = ch;
-    if (ws_need(L, dbl, (int)p->rpad, false) + extra > ext_bytes)
+    if (ws_need(L, dbl, (int)p->rpad, false) + sep_b > ext_bytes)
       return fail(FST_EINVAL, "signal too long for the fixed scratch buffer");
   }
   return run_conv<T>(p->R, L, a, npairs, ext_ws);
@@ -858,6 +931,10 @@ static fst_status plan_end(fst_plan_t p, double *S, const std::vector<double> &l
       if ((s = R->zero(p->ST32, nst * sizeof(float))) != FST_OK) return bail(s);
     }
     if ((s = R->to_f32(p->D64, p->D32, p->rpad)) != FST_OK) return bail(s);
+    std::vector<unsigned char> par(p->rpad, 0);
+    for (int64_t j = 0; j < p->r; ++j) par[j] = (unsigned char)(p->idx[j] & 1);
+    if ((s = R->alloc((void **)&p->cpar, par.size())) != FST_OK) return bail(s);
+    if ((s = R->h2d(p->cpar, par.data(), par.size())) != FST_OK) return bail(s);
     if ((s = R->alloc((void **)&p->ST32_hl, nst * sizeof(float2))) != FST_OK) return bail(s);
     if ((s = R->split_tf32(p->ST32, p->ST32_hl, (int64_t)nst)) != FST_OK) return bail(s);
     if ((s = R->sync()) != FST_OK) return bail(s);
@@ -956,7 +1033,7 @@ void destroy_plan(fst_plan_t p) {
     R->sync();
     for (auto &e : p->graphs) R->graph_destroy(e.exec);
     p->graphs.clear();
-    void *bufs[] = {p->spec32, p->ST32, p->D32, p->spec64, p->ST64, p->D64, p->ST32_hl, p->STt, p->spec_unit,
+    void *bufs[] = {p->spec32, p->ST32, p->D32, p->spec64, p->ST64, p->D64, p->ST32_hl, p->STt, p->spec_unit, p->cpar,
                     p->tw32h, p->tw32l, p->tw64h, p->tw64l, p->twB, p->tw8, p->ws};
     for (void *b : bufs)
       if (b) R->release(b);

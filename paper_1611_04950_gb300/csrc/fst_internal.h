@@ -72,6 +72,12 @@ struct Runner {
   virtual fst_status passB(const ConvArgs<double> &a, const Layout &L) = 0;
   virtual fst_status passC(const ConvArgs<float> &a, const Layout &L) = 0;
   virtual fst_status passC(const ConvArgs<double> &a, const Layout &L) = 0;
+  // FP64 four-step passes of fst_fast64.cuh (device): a.log2P, log2Q, Pnz, inter, ... set
+  virtual fst_status f64_passes(const ConvArgs<double> &a, int spec_log2P, int pass) { return FST_EUNSUPPORTED; }
+  virtual fst_status f64_corr(const ConvArgs<double> &a, const unsigned char *cpar, int64_t rows, int chunk,
+                              double *part, double *acoef) { return FST_EUNSUPPORTED; }
+  virtual fst_status f64_z(const ConvArgs<double> &a, const unsigned char *cpar, int64_t rows,
+                           const double *acoef) { return FST_EUNSUPPORTED; }
   // ragged batch: one single-CTA transform per descriptor (all with FFT length 2^base.log2M)
   virtual fst_status small_ragged(const RaggedDesc<float> *d, int count, const ConvArgs<float> &base,
                                   const Layout &L) = 0;
@@ -179,6 +185,7 @@ struct fst_plan_s {
   int tc_nB = 0;
   int64_t tc_Npad = 0;
   double *spec64 = nullptr, *ST64 = nullptr, *D64 = nullptr;
+  unsigned char *cpar = nullptr;   // [rpad] 1: column j of S_T antisymmetric (its index is odd)
   double *spec_unit = nullptr;   // plan-time only: DFT_M(c) / M for the eigenvalues
   float2 *tw32h = nullptr, *tw32l = nullptr;
   // stage twiddles of the 4096-point row FFT: [t][k] = W_256^{k t} (k < 16), then

@@ -1,0 +1,41 @@
+"""FP64 four-step kernels (fst_fast64.cuh) at the sizes where they can go wrong: every split of M =
+2^10 .. 2^18 (P = 8, 16, 32; 32- to 8192-point rows), odd and ragged lengths, odd batches, complex
+signals, ranks above one shared-memory round, in place, strided.  Against the FP64 oracle; tolerance
+1e-12 of ||y||, the FP64 tolerance of the parity tests."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+from paper_1611_04950_gb300 import fst as F  # noqa: E402
+from paper_1611_04950_gb300 import workloads  # noqa: E402
+from oracle import fst_oracle as O  # noqa: E402
+
+
+@pytest.mark.parametrize("N,W,eps,K,batch,cplx", [
+    (511, 0.2, 1e-6, None, 3, False), (257, 0.1, 1e-3, None, 1, True), (1000, 1 / 64, 1e-8, None, 5, False),
+    (2047, 0.25, 1e-8, None, 9, True), (4096, 1 / 16, 1e-6, None, 2, False), (4097, 0.2, 1e-6, None, 33, False),
+    (8191, 0.05, 1e-4, None, 2, True), (9001, 0.1, 1e-6, None, 7, False), (20011, 0.25, 1e-8, None, 3, True),
+    (65536, 1 / 8, 1e-4, None, 5, False), (100003, 0.03, 1e-6, None, 2, True), (600, 0.2, 1e-6, 40, 17, False)])
+def test_fp64_against_oracle(N, W, eps, K, batch, cplx):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    p = F.Plan(N, W, K=K, eps=eps)
+    o = O.make_plan(N, W, p.K, eps)
+    assert p.r == o.r
+    y = workloads.gaussian(batch, N, seed=N, complex_=cplx)
+    nrm = np.linalg.norm(y.numpy(), axis=1)
+    ref = O.fast_project(o, y.numpy().T).T
+    yd = y.to("cuda")
+    out = p.project(yd)
+    assert np.all(np.linalg.norm(out.cpu().numpy() - ref, axis=1) < 1e-12 * nrm)
+    assert torch.equal(p.project(yd), out)
+    wide = torch.zeros((batch, N + 5), dtype=y.dtype, device="cuda")
+    wide[:, :N] = yd
+    got = p.project(wide[:, :N], out=wide[:, :N])          # in place, strided rows
+    assert torch.equal(got, out) and torch.count_nonzero(wide[:, N:]) == 0
+    b = p.apply_prolate(yd).cpu().numpy()
+    z = (o.S_T @ (o.D[:, None] * (o.S_T.T @ y.numpy().T))).T
+    assert np.all(np.linalg.norm(b + z - ref, axis=1) < 1e-12 * nrm)
