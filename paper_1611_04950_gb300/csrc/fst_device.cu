@@ -19,6 +19,7 @@
 #include "fst_fast.cuh"
 #include "fst_big.cuh"
 #include "fst_fast64.cuh"
+#include "fst_small32.cuh"
 #define FST_TC_KERNELS
 #include "fst_tc.cuh"
 
@@ -474,6 +475,10 @@ static fst_status set_attrs() {
   CU(cudaFuncSetAttribute(k_passB<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
   CU(cudaFuncSetAttribute(k_passC<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
   CU(cudaFuncSetAttribute(k_passC<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
+  CU(cudaFuncSetAttribute(k_small32<13>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_smem(13, SM_RMAX)), "attr");
+  CU(cudaFuncSetAttribute(k_small32<14>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_smem(14, SM_RMAX)), "attr");
+  CU(cudaFuncSetAttribute(k_small32_ragged<13>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_smem(13, SM_RMAX)), "attr");
+  CU(cudaFuncSetAttribute(k_small32_ragged<14>, cudaFuncAttributeMaxDynamicSharedMemorySize, sm_smem(14, SM_RMAX)), "attr");
   CU(cudaFuncSetAttribute(k_fastAw<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, fastw_smem(32)), "attr");
   CU(cudaFuncSetAttribute(k_fastAw<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, fastw_smem(16)), "attr");
   CU(cudaFuncSetAttribute(k_fastAw<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, fastw_smem(8)), "attr");
@@ -799,7 +804,58 @@ struct DevRunner : Runner {
                           const Layout &L) override { return small_ragged_t(d, count, base, L); }
   fst_status small_ragged(const RaggedDesc<double> *d, int count, const ConvArgs<double> &base,
                           const Layout &L) override { return small_ragged_t(d, count, base, L); }
-  fst_status small(const ConvArgs<float> &a, const Layout &L) override { return small_t(a, L); }
+  template <int LM> fst_status small32_t(const ConvArgs<float> &a) {
+    TRY(set_attrs());
+    SmallPlan p{a.spec, a.ST, a.STt, a.D, a.twS, a.tc_Npad, (int)a.N, a.r, a.rpad, {a.odd[0], a.odd[1], a.odd[2], a.odd[3]}};
+    PROF("k_small32", a.npairs, (k_small32<LM><<<(unsigned)a.npairs, (1 << LM) / 16, sm_smem(LM, a.rpad), cur>>>(a, p)));
+    LAUNCHED("k_small32");
+    return FST_OK;
+  }
+  template <int LM>
+  fst_status small32_ragged_t(const SmallDesc *d, int count, int rpad_max, const float2 *twB, int cplx) {
+    TRY(set_attrs());
+    PROF("k_small32_ragged", count,
+         (k_small32_ragged<LM><<<(unsigned)count, (1 << LM) / 16, sm_smem(LM, rpad_max), cur>>>(d, twB, cplx)));
+    LAUNCHED("k_small32_ragged");
+    return FST_OK;
+  }
+  fst_status small32_prep(const Tw<double> &tw, int log2M, float2 *twS, const float *ST, int64_t N, int rpad, int r,
+                          float *STs) override {
+    if (sm_words(log2M) > 0) {
+      k_tw_small<<<grid_for(sm_words(log2M), 256), 256, 0, s>>>(tw, log2M, twS);
+      LAUNCHED("k_tw_small");
+    }
+    if (r > 0) {
+      k_tc_prep<<<grid_for(r * N, 256), 256, 0, s>>>(ST, N, rpad, r, r, N, STs);
+      LAUNCHED("k_tc_prep");
+    }
+    return FST_OK;
+  }
+  fst_status small32_ragged(const SmallDesc *d, int count, int log2M, int rpad_max, const float2 *twB,
+                            int cplx) override {
+    switch (log2M) {
+      case 10: return small32_ragged_t<10>(d, count, rpad_max, twB, cplx);
+      case 11: return small32_ragged_t<11>(d, count, rpad_max, twB, cplx);
+      case 12: return small32_ragged_t<12>(d, count, rpad_max, twB, cplx);
+      case 13: return small32_ragged_t<13>(d, count, rpad_max, twB, cplx);
+      case 14: return small32_ragged_t<14>(d, count, rpad_max, twB, cplx);
+      default: return fail(FST_EINVAL, "single-CTA transform length out of range");
+    }
+  }
+  fst_status small(const ConvArgs<float> &a, const Layout &L) override {
+    // the restructured kernel where its tables exist (M = 2^10 .. 2^14, r <= 128)
+    if (a.twS && (a.mode == MODE_FULL || a.mode == MODE_CONV)) {
+      switch (a.log2M) {
+        case 10: return small32_t<10>(a);
+        case 11: return small32_t<11>(a);
+        case 12: return small32_t<12>(a);
+        case 13: return small32_t<13>(a);
+        case 14: return small32_t<14>(a);
+        default: break;
+      }
+    }
+    return small_t(a, L);
+  }
   fst_status small(const ConvArgs<double> &a, const Layout &L) override { return small_t(a, L); }
   template <int P2> fst_status colA_t(const ConvArgs<float> &a, const Layout &L) {
     TRY(set_attrs());

@@ -280,6 +280,13 @@ static fst_status ensure_ws(fst_plan_t p, size_t bytes) {
   return FST_OK;
 }
 
+// antisymmetric columns of S_T as bits (r <= 128)
+static void odd_bits(fst_plan_t p, unsigned *odd) {
+  for (int w = 0; w < 4; ++w) odd[w] = 0;
+  for (int j = 0; j < (int)std::min<int64_t>(p->r, 128); ++j)
+    if (p->idx[j] & 1) odd[j >> 5] |= 1u << (j & 31);
+}
+
 // FP64 four-step path of fst_fast64.cuh: M = 2^10 .. 2^18.  The split is P = 32, or for batches whose
 // rows fill the GPU that of the plan's FP64 layout (rows of at least 2048 points, the faster row
 // kernel).  The plan's spectrum keeps its own order (natural up to M = 2^13).
@@ -372,6 +379,12 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
     a.tc_Npad = p->tc_Npad;
     a.twB = p->twB;
     a.tw8 = p->tw8;
+    if (p->twS) {
+      a.twS = p->twS;
+      a.STt = p->STs;
+      a.tc_Npad = p->N;
+      odd_bits(p, a.odd);
+    }
   }
   a.r = full ? (int)p->r : 0;
   a.rpad = (int)p->rpad;
@@ -952,6 +965,14 @@ static fst_status plan_end(fst_plan_t p, double *S, const std::vector<double> &l
       return bail(s);
     if ((s = R->sync()) != FST_OK) return bail(s);
   }
+  if (R->device() && p->lay32.small && p->log2M >= 10 && p->rpad <= SM_RMAX) {
+    fst_status s;
+    if ((s = R->alloc((void **)&p->twS, (size_t)std::max(1, sm_words(p->log2M)) * sizeof(float2))) != FST_OK) return bail(s);
+    if ((s = R->alloc((void **)&p->STs, (size_t)std::max<int64_t>(1, p->r * N) * sizeof(float))) != FST_OK) return bail(s);
+    if ((s = R->small32_prep(plan_tw<double>(p), p->log2M, p->twS, p->ST32, N, (int)p->rpad, (int)p->r, p->STs)) != FST_OK)
+      return bail(s);
+    if ((s = R->sync()) != FST_OK) return bail(s);
+  }
   if (p->lay32.small && p->lay32.smem_small > 227 * 1024)
     return bail(fail(FST_EUNSUPPORTED, "transition rank too large for the single-CTA path"));
   if (p->lay64.small && p->lay64.smem_small > 227 * 1024)
@@ -1033,7 +1054,7 @@ void destroy_plan(fst_plan_t p) {
     R->sync();
     for (auto &e : p->graphs) R->graph_destroy(e.exec);
     p->graphs.clear();
-    void *bufs[] = {p->spec32, p->ST32, p->D32, p->spec64, p->ST64, p->D64, p->ST32_hl, p->STt, p->spec_unit, p->cpar,
+    void *bufs[] = {p->spec32, p->ST32, p->D32, p->spec64, p->ST64, p->D64, p->ST32_hl, p->STt, p->spec_unit, p->cpar, p->twS, p->STs,
                     p->tw32h, p->tw32l, p->tw64h, p->tw64l, p->twB, p->tw8, p->ws};
     for (void *b : bufs)
       if (b) R->release(b);
@@ -1922,6 +1943,31 @@ static fst_status ragged_t(const fst_plan_t *plans, const void *const *y, void *
     Runner *R = p0->R;
     Layout L = make_layout(p0->N, lg, dbl, maxr[lg], false);
     void *dd = nullptr;
+    // FP32 device plans with the single-CTA tables: the restructured kernel
+    std::vector<SmallDesc> sd;
+    for (int64_t i = 0; !dbl && i < count; ++i) {
+      fst_plan_t p = plans[i];
+      if (p->log2M != lg || !p->lay32.small || !p->twS) continue;
+      SmallDesc q{};
+      q.y = (const float *)y[i];
+      q.out = (float *)out[i];
+      q.p.spec = p->spec32;
+      q.p.ST = p->ST32;
+      q.p.STt = p->STs;
+      q.p.D = p->D32;
+      q.p.twS = p0->twS;   // the same table for every plan of the length: it stays in L2
+      q.p.ld_t = p->N;
+      q.p.N = (int)p->N;
+      q.p.r = (int)p->r;
+      q.p.rpad = (int)p->rpad;
+      odd_bits(p, q.p.odd);
+      sd.push_back(q);
+    }
+    if (sd.size() == buckets[lg].size()) {
+      TRY(ragged_buf(R, st, sd.size() * sizeof(SmallDesc), sd.data(), &dd));
+      TRY(R->small32_ragged((const SmallDesc *)dd, (int)sd.size(), lg, maxr[lg], p0->twB, cplx ? 1 : 0));
+      continue;
+    }
     TRY(ragged_buf(R, st, buckets[lg].size() * sizeof(RaggedDesc<T>), buckets[lg].data(), &dd));
     ConvArgs<T> base{};
     base.batch = 1;

@@ -83,6 +83,11 @@ struct Runner {
                                   const Layout &L) = 0;
   virtual fst_status small_ragged(const RaggedDesc<double> *d, int count, const ConvArgs<double> &base,
                                   const Layout &L) = 0;
+  // FP32 single-CTA path (device): stage twiddles and the K-major copy of S_T; ragged launch
+  virtual fst_status small32_prep(const Tw<double> &tw, int log2M, float2 *twS, const float *ST, int64_t N, int rpad,
+                                  int r, float *STs) { return FST_EUNSUPPORTED; }
+  virtual fst_status small32_ragged(const SmallDesc *d, int count, int log2M, int rpad_max, const float2 *twB,
+                                    int cplx) { return FST_EUNSUPPORTED; }
   // separate correction (FP32, device): partials, reduce to a = D o c, out += S_T a
   virtual fst_status corr_c(const ConvArgs<float> &a) { return FST_EUNSUPPORTED; }
   // tcgen05 S_T^T y over every pair of a (a.pair0 = 0): partials [pair][a.nkb][2][rpad]
@@ -191,6 +196,8 @@ struct fst_plan_s {
   // stage twiddles of the 4096-point row FFT: [t][k] = W_256^{k t} (k < 16), then
   // W_4096^{k t} (k < 256), t < 16
   float2 *twB = nullptr;
+  float2 *twS = nullptr;   // single-CTA path: its stage twiddles (device plans, M = 2^10 .. 2^14), and
+  float *STs = nullptr;    // the K-major copy of S_T, [r][N]
   float2 *tw8 = nullptr;   // stage twiddles of the 8192-point row FFT (FP64 built)
   double2 *tw64h = nullptr, *tw64l = nullptr;
   void *ws = nullptr;

@@ -137,6 +137,8 @@ template <typename T> struct ConvArgs {
   int64_t tc_Npad;
   const float2 *twB;  // FP32 device plans: stage twiddles of the 4096-point row FFT, then W_1024^t
   const float2 *tw8;  // FP32 device plans: stage twiddles of the 8192-point row FFT
+  const float2 *twS;  // FP32 device plans of the single-CTA path: stage twiddles, S_T's antisymmetric
+  unsigned odd[4];    // columns as bits (STt then holds its K-major copy, rows tc_Npad apart)
   const RPair<T> *rp; // ragged batch: per pair slot signal, length and spectrum (else nullptr)
   int two_spec;       // ragged real slots hold two signals with their own spectra (pass B pairs rows)
 };
@@ -166,6 +168,38 @@ template <typename T> struct RaggedDesc {
   const T *D;
   int64_t N;
   int r, rpad;
+};
+
+// ---- FP32 single-CTA projection (fst_small32.cuh, device) ----
+// stage twiddles of the inverse radix-16 stages at Ns = R0 16^i, [t][k] W_{16 Ns}^{k t}, then (R0 > 1)
+// the forward radix-R0 stage, [t - 1][j] W_M^{j t}, j < M / R0
+__host__ __device__ constexpr int sm_r0(int log2M) { return 1 << (log2M & 3); }
+__host__ __device__ constexpr int sm_n16(int log2M) { return log2M >> 2; }
+__host__ __device__ constexpr int sm_off(int log2M, int i) {   // of inverse stage i (i = n16: the forward stage)
+  int o = 0, ns = sm_r0(log2M);
+  for (int q = 0; q < i; ++q, ns *= 16) o += 16 * ns;
+  return o;
+}
+__host__ __device__ constexpr int sm_words(int log2M) {
+  return sm_off(log2M, sm_n16(log2M)) + (sm_r0(log2M) - 1) * ((1 << log2M) / sm_r0(log2M));
+}
+constexpr int SM_RMAX = 128;
+
+struct SmallPlan {
+  const float *spec;      // natural order
+  const float *ST;        // [N][rpad]
+  const float *STt;       // [.][ld_t]
+  const float *D;
+  const float2 *twS;
+  int64_t ld_t;
+  int N, r, rpad;
+  unsigned odd[4];
+};
+// a signal of a ragged batch with its plan's data
+struct SmallDesc {
+  const float *y;
+  float *out;
+  SmallPlan p;
 };
 
 template <typename T> struct KState {
