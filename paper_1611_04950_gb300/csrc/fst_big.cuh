@@ -29,8 +29,9 @@ template <bool INV> __device__ __forceinline__ float2 big_wP(const ConvArgs<floa
 // ---------------------------------------------------------------------------
 // pass A: grid (Q / NB, npairs), 256 threads, dynamic shared memory big_smem_bytes(P2)
 // ---------------------------------------------------------------------------
-template <int P2>
-__global__ void __launch_bounds__(256, 3) k_colA(const ConvArgs<float> a) {
+// FULL: a full-length forward transform (no zero rows)
+template <int P2, bool FULL = false>
+__global__ void __launch_bounds__(256, FULL ? 2 : 3) k_colA(const ConvArgs<float> a) {
   constexpr int NB = big_nb(P2), BS = big_bs(P2), P = 32 * P2;
   extern __shared__ __align__(16) float2 bsm[];
   const int Q = 1 << a.log2Q;
@@ -40,16 +41,18 @@ __global__ void __launch_bounds__(256, 3) k_colA(const ConvArgs<float> a) {
   const int col = threadIdx.x % NB, hi = threadIdx.x / NB;   // hi: b in stage 1, k group in stage 2
   const int64_t n2 = n2_0 + col;
   {
-    // stage 1: b = hi; x[P2 a + b] for a < 16
+    // stage 1: b = hi; x[P2 a + b] for a < 16 (FULL: a < 32)
     const int b = hi;
     float2 v[32];
 #pragma unroll
-    for (int q = 0; q < 16; ++q) {
+    for (int q = 0; q < (FULL ? 32 : 16); ++q) {
       const int n1 = P2 * q + b;
       const int64_t n = (int64_t)n1 * Q + n2;
-      v[q] = (n1 < a.Pnz && n < a.N) ? load_pair(a, pl, n) : make_float2(0.f, 0.f);
+      if (FULL) v[q] = load_full(a, pl, n);
+      else v[q] = (n1 < a.Pnz && n < a.N) ? load_pair(a, pl, n) : make_float2(0.f, 0.f);
     }
-    dft_half_in<32>(v);
+    if (FULL) RegDft<32, false>::run(v);
+    else dft_half_in<32>(v);
     float2 *s = bsm + b * BS + col;
     s[0] = v[0];
 #pragma unroll
@@ -59,7 +62,7 @@ __global__ void __launch_bounds__(256, 3) k_colA(const ConvArgs<float> a) {
   // stage 2: tasks k = hi + P2 i; outputs k1 = k + 32 m, times W_M^{n2 k1}
   float2 *dst = a.inter + (pl * P) * (int64_t)Q + n2;
   // W_M^{n2 (k + 32 m)} = alpha_k beta^m, beta = W_M^{32 n2}: every 8th m from an exact lookup
-  // of W_M^{n2 (k + 32 m)}, the others by at most 7 products with beta
+  // of W_M^{n2 (k + 32 m)}, the others by at most 7 products with beta (FULL: every m looked up)
   const float2 beta = a.tw.root<false>(32 * (uint64_t)n2, a.log2M);
 #pragma unroll 2
   for (int i = 0; i < 32 / P2; ++i) {
@@ -71,7 +74,7 @@ __global__ void __launch_bounds__(256, 3) k_colA(const ConvArgs<float> a) {
     float2 t;
 #pragma unroll
     for (int m = 0; m < P2; ++m) {
-      if ((m & 7) == 0) t = a.tw.root<false>((uint64_t)n2 * (uint64_t)(k + 32 * m), a.log2M);
+      if (FULL || (m & 7) == 0) t = a.tw.root<false>((uint64_t)n2 * (uint64_t)(k + 32 * m), a.log2M);
       else t = cmul(t, beta);
       dst[(int64_t)(k + 32 * m) * Q] = (k == 0 && m == 0) ? u[0] : cmul(u[m], t);
     }

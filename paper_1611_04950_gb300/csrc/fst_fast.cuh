@@ -177,6 +177,26 @@ __device__ __forceinline__ void fastA_finish(const ConvArgs<float> &a, float2 *v
 }
 
 // ---------------------------------------------------------------------------
+// pass A of a full-length forward transform (T2^* y, T1 c: no zero rows), one column per thread.
+// Bound: memory; every load and store is coalesced along the columns.
+// grid (Q / 256, pairs), 256 threads
+// ---------------------------------------------------------------------------
+template <int P> __global__ void __launch_bounds__(256) k_fastA_full(const ConvArgs<float> a) {
+  const int Q = 1 << a.log2Q;
+  const int64_t pl = blockIdx.y, n2 = (int64_t)blockIdx.x * 256 + threadIdx.x;
+  float2 v[P];
+#pragma unroll
+  for (int n1 = 0; n1 < P; ++n1) v[n1] = load_full(a, pl, (int64_t)n1 * Q + n2);
+  RegDft<P, false>::run(v);
+  // every factor from the tables (products of a few powers, as fastA_finish forms them, would
+  // lose accuracy that this memory-bound pass need not give up)
+  float2 *dst = a.inter + (pl * P) * (int64_t)Q + n2;
+#pragma unroll
+  for (int k1 = 0; k1 < P; ++k1)
+    dst[(int64_t)k1 * Q] = k1 == 0 ? v[0] : cmul(v[k1], a.tw.root<false>((uint64_t)n2 * (uint64_t)k1, a.log2M));
+}
+
+// ---------------------------------------------------------------------------
 // pass A without the correction (B y alone, or a = D o S_T^T y computed beforehand), real
 // signals: tiles of FASTW_G pairs x FASTW_NB columns, so each warp load reads 256 contiguous
 // bytes of a signal row; the tile is transposed through shared memory to one column per

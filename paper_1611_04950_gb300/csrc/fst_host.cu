@@ -1368,7 +1368,8 @@ static fst_status coeffs_t(fst_plan_t p, const T *y, c2<T> *out, int64_t batch, 
   int log2N = 0;
   while ((1LL << log2N) < N) ++log2N;
   // ---- F^* y: forward DFT of length N, chunk by chunk of pairs, then the bins
-  Layout Lf = make_layout(N, log2N, dbl, 0, false);
+  // FP32 device plans: register column passes and the 4096-point row kernel, without zero rows
+  Layout Lf = make_layout(N, log2N, dbl, 0, !dbl && R->device());
   if (!Lf.small) Lf.Pnz = 1 << Lf.log2P;
   const int64_t npairs = cplx ? batch : (batch + 1) / 2;
   const size_t ws_f = ws_need(Lf, dbl, 0, true) + 4096;
@@ -1389,6 +1390,8 @@ static fst_status coeffs_t(fst_plan_t p, const T *y, c2<T> *out, int64_t batch, 
     a.r = 0;
     a.rpad = 0;
     a.tw = plan_tw<T>(p);
+    a.twB = p->twB;
+    a.tw8 = p->tw8;
     a.mode = MODE_FORWARD;
     a.log2M = Lf.log2M;
     a.log2P = Lf.log2P;
@@ -1501,10 +1504,12 @@ static fst_status expand_t(fst_plan_t p, const c2<T> *coef, c2<T> *out, int64_t 
   const bool dbl = sizeof(T) == 8;
   int log2N = 0;
   while ((1LL << log2N) < N) ++log2N;
-  Layout Lf = make_layout(N, log2N, dbl, 0, false);
+  Layout Lf = make_layout(N, log2N, dbl, 0, !dbl && R->device());
   if (!Lf.small) Lf.Pnz = 1 << Lf.log2P;
-  // scratch: the scattered rows of one launch group, then the forward transform's own
-  const size_t xs_b = ((size_t)Lf.chunk * N * sizeof(C) + 255) / 256 * 256;
+  // FP32 device plans: the column pass reads the coefficients itself; otherwise the scattered rows
+  // of one launch group come first in the scratch
+  const bool direct = Lf.fast || Lf.big;
+  const size_t xs_b = direct ? 0 : ((size_t)Lf.chunk * N * sizeof(C) + 255) / 256 * 256;
   TRY(ensure_ws(p, xs_b + ws_need(Lf, dbl, 0, true) + 4096));
   C *Xs = (C *)p->ws;
   char *wf = (char *)p->ws + xs_b;
@@ -1527,6 +1532,12 @@ static fst_status expand_t(fst_plan_t p, const c2<T> *coef, c2<T> *out, int64_t 
   a.cplx = 1;
   a.N = N;
   a.tw = plan_tw<T>(p);
+  a.twB = p->twB;
+  a.tw8 = p->tw8;
+  if (direct) {
+    a.exp_kp = e.Kp;
+    a.exp_h = e.h;
+  }
   a.mode = MODE_FORWARD;
   a.log2M = Lf.log2M;
   a.log2P = Lf.log2P;
@@ -1542,7 +1553,8 @@ static fst_status expand_t(fst_plan_t p, const c2<T> *coef, c2<T> *out, int64_t 
   for (int64_t s0 = 0; s0 < batch; s0 += Lf.chunk) {
     const int64_t nsig = std::min<int64_t>(Lf.chunk, batch - s0);
     e.sig0 = s0;
-    TRY(R->exp_scatter(e, nsig, Xs));
+    if (direct) a.exp_c = coef + s0 * e.Kp;
+    else TRY(R->exp_scatter(e, nsig, Xs));
     a.batch = nsig;
     a.pair0 = 0;
     a.npairs = nsig;

@@ -139,6 +139,8 @@ template <typename T> struct ConvArgs {
   const float2 *tw8;  // FP32 device plans: stage twiddles of the 8192-point row FFT
   const float2 *twS;  // FP32 device plans of the single-CTA path: stage twiddles, S_T's antisymmetric
   unsigned odd[4];    // columns as bits (STt then holds its K-major copy, rows tc_Npad apart)
+  const c2<T> *exp_c; // forward transform of T1 c: coefficient vectors, exp_kp apart, bins -exp_h..exp_h first
+  int64_t exp_kp, exp_h;
   const RPair<T> *rp; // ragged batch: per pair slot signal, length and spectrum (else nullptr)
   int two_spec;       // ragged real slots hold two signals with their own spectra (pass B pairs rows)
 };
@@ -242,6 +244,15 @@ template <typename T> FST_HD void store_pair(const ConvArgs<T> &a, int64_t pl, i
   const int64_t s0 = 2 * p, s1 = 2 * p + 1;
   a.out[s0 * a.ld + n] = v.x;
   if (s1 < a.batch) a.out[s1 * a.ld + n] = v.y;
+}
+
+// input n < N of a full-length forward transform: a signal pair's sample, or (T1 c) the conjugate of
+// the coefficient at the bin n (n <= h) or n - N (n >= N - h), zero elsewhere
+template <typename T> FST_HD c2<T> load_full(const ConvArgs<T> &a, int64_t pl, int64_t n) {
+  if (!a.exp_c) return load_pair(a, pl, n);
+  const int64_t k = n <= a.exp_h ? n : n - a.N;
+  if (k < -a.exp_h || k > a.exp_h) return mk<T>(0, 0);
+  return cconj(a.exp_c[(a.pair0 + pl) * a.exp_kp + k + a.exp_h]);
 }
 
 // spectrum of local pair pl (its own for a ragged batch)
