@@ -301,14 +301,19 @@ FST_HD void coef_gather_body(const c2<T> *X, const Layout &Lf, int64_t N, int cp
 // totals[sig][o] = sum over chunks (fixed order) of part[sig][chunk][o]
 template <typename T>
 FST_HD void coef_reduce_body(const T *part, int nchunks, int nout, int64_t sig, int o, T *tot) {
-  T sr = 0, si = 0;
-  for (int c = 0; c < nchunks; ++c) {
-    const T *q = part + ((sig * nchunks + c) * (int64_t)nout + o) * 2;
-    sr += q[0];
-    si += q[1];
+  // eight interleaved chains: their loads overlap, and the chains of roundings are short
+  T sr[8] = {0, 0, 0, 0, 0, 0, 0, 0}, si[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  for (int c0 = 0; c0 < nchunks; c0 += 8) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+      if (c0 + i < nchunks) {
+        const T *q = part + ((sig * nchunks + c0 + i) * (int64_t)nout + o) * 2;
+        sr[i] += q[0];
+        si[i] += q[1];
+      }
   }
-  tot[(sig * (int64_t)nout + o) * 2] = sr;
-  tot[(sig * (int64_t)nout + o) * 2 + 1] = si;
+  tot[(sig * (int64_t)nout + o) * 2] = ((sr[0] + sr[1]) + (sr[2] + sr[3])) + ((sr[4] + sr[5]) + (sr[6] + sr[7]));
+  tot[(sig * (int64_t)nout + o) * 2 + 1] = ((si[0] + si[1]) + (si[2] + si[3])) + ((si[4] + si[5]) + (si[6] + si[7]));
 }
 
 // final L2^* y and U2^* y entries (index o in [0, r1 + r)) from the raw totals

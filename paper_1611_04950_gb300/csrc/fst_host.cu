@@ -1373,13 +1373,17 @@ static fst_status coeffs_t(fst_plan_t p, const T *y, c2<T> *out, int64_t batch, 
   if (!Lf.small) Lf.Pnz = 1 << Lf.log2P;
   const int64_t npairs = cplx ? batch : (batch + 1) / 2;
   const size_t ws_f = ws_need(Lf, dbl, 0, true) + 4096;
-  const int nchunks = (int)((N + COEF_CHUNK - 1) / COEF_CHUNK);
+  // FP32 on the device: all signals share the generated columns
+  size_t lr_b = 0;
+  const int lr_chunks = dbl ? 0 : R->lowrank_plan(N, cp->rH, cp->DA, cp->DB, cplx ? 2 * batch : batch, &lr_b);
+  const int schunks = (int)((N + COEF_CHUNK - 1) / COEF_CHUNK);
+  const int nchunks = lr_chunks > 0 ? lr_chunks : schunks;
   const size_t part_b = (size_t)batch * nchunks * cp->nraw * 2 * sizeof(T);
-  const size_t partU_b = std::max((size_t)batch * nchunks * std::max<int64_t>(p->r, 1) * 2 * sizeof(T),
+  const size_t partU_b = std::max((size_t)batch * schunks * std::max<int64_t>(p->r, 1) * 2 * sizeof(T),
                                   split_corr_bytes(N, npairs, (int)p->rpad));
   const size_t tot_b = (size_t)batch * cp->nraw * 2 * sizeof(T);
   const size_t totU_b = (size_t)batch * std::max<int64_t>(p->r, 1) * 2 * sizeof(T);
-  TRY(ensure_ws(p, std::max(ws_f, part_b + partU_b + tot_b + totU_b + 4096)));
+  TRY(ensure_ws(p, std::max(ws_f, part_b + partU_b + tot_b + totU_b + 4096 + lr_b)));
   {
     ConvArgs<T> a{};
     a.y = y;
@@ -1441,7 +1445,12 @@ static fst_status coeffs_t(fst_plan_t p, const T *y, c2<T> *out, int64_t batch, 
   c.rpad = (int)p->rpad;
   const T *CA, *CB, *sq;
   CoefPtrs<T>::fill(cp, c, CA, CB, sq);
-  TRY(R->coef_lowrank(c));
+  if (lr_chunks > 0) {
+    const size_t at = (part_b + partU_b + tot_b + totU_b + 255) / 256 * 256;
+    TRY(R->coef_gemm(*reinterpret_cast<const CoefArgs<float> *>(&c), w + at));
+  } else {
+    TRY(R->coef_lowrank(c));
+  }
   const bool mma_u = !dbl && R->device() && p->r > 0;
   if (mma_u) {
     // U2^* y on the tensor cores: S_T^T y per pair, scaled by sqrt|D| in the reduce
@@ -1467,10 +1476,12 @@ static fst_status coeffs_t(fst_plan_t p, const T *y, c2<T> *out, int64_t batch, 
     c.upairs = 1;
     c.acoefU = (const T *)ca.acoef;
   } else if (p->r > 0) {
+    c.nchunks = schunks;
     TRY(R->coef_st(c));
+    c.nchunks = nchunks;
   }
   TRY(R->coef_reduce(c.part, nchunks, cp->nraw, batch, tot));
-  if (p->r > 0 && !mma_u) TRY(R->coef_reduce(c.partU, nchunks, (int)p->r, batch, totU));
+  if (p->r > 0 && !mma_u) TRY(R->coef_reduce(c.partU, schunks, (int)p->r, batch, totU));
   TRY(R->coef_mix(c, tot, totU, CA, CB, sq, out, Kp, nF));
   return FST_OK;
 }
@@ -1510,7 +1521,9 @@ static fst_status expand_t(fst_plan_t p, const c2<T> *coef, c2<T> *out, int64_t 
   // of one launch group come first in the scratch
   const bool direct = Lf.fast || Lf.big;
   const size_t xs_b = direct ? 0 : ((size_t)Lf.chunk * N * sizeof(C) + 255) / 256 * 256;
-  TRY(ensure_ws(p, xs_b + ws_need(Lf, dbl, 0, true) + 4096));
+  const size_t fwd_b = (ws_need(Lf, dbl, 0, true) + 4096) / 256 * 256;
+  const size_t lr_b = dbl ? 0 : R->expand_scratch(N, cp->rH, cp->DA, cp->DB, (int)p->r, std::min<int64_t>(Lf.chunk, batch));
+  TRY(ensure_ws(p, xs_b + fwd_b + lr_b));
   C *Xs = (C *)p->ws;
   char *wf = (char *)p->ws + xs_b;
   ExpArgs<T> e{};
@@ -1565,7 +1578,8 @@ static fst_status expand_t(fst_plan_t p, const c2<T> *coef, c2<T> *out, int64_t 
       TRY(R->passB(a, Lf));
     }
     e.X = (const C *)a.inter;
-    TRY(R->expand(e, nsig));
+    if (lr_b) TRY(R->expand_gemm(*reinterpret_cast<const ExpArgs<float> *>(&e), nsig, wf + fwd_b, p->cpar));
+    else TRY(R->expand(e, nsig));
   }
   return FST_OK;
 }

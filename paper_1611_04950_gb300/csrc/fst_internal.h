@@ -140,6 +140,14 @@ struct Runner {
   virtual fst_status to_f32(const double *src, float *dst, int64_t n) = 0;
   virtual fst_status split_tf32(const float *src, float2 *hl, int64_t n) = 0;
 
+  // FP32 low-rank sums and T1 c with shared columns (fst_lowrank.cuh, device): the number of sample
+  // chunks and bytes of scratch they want (0 chunks: not for these sizes), then the launches
+  virtual int lowrank_plan(int64_t N, int rH, int DA, int DB, int64_t nvc, size_t *scratch) { return 0; }
+  virtual fst_status coef_gemm(const CoefArgs<float> &a, void *scratch) { return FST_EUNSUPPORTED; }
+  virtual size_t expand_scratch(int64_t N, int rH, int DA, int DB, int r, int64_t nsig) { return 0; }
+  virtual fst_status expand_gemm(const ExpArgs<float> &a, int64_t nsig, void *scratch, const unsigned char *cpar) {
+    return FST_EUNSUPPORTED;
+  }
   // fast coefficient vector kernels (runner memory)
   virtual fst_status coef_lowrank(const CoefArgs<float> &a) = 0;
   virtual fst_status coef_lowrank(const CoefArgs<double> &a) = 0;
