@@ -21,6 +21,7 @@
 #include "fst_fast64.cuh"
 #include "fst_small32.cuh"
 #include "fst_lowrank.cuh"
+#include "fst_sym.cuh"
 #define FST_TC_KERNELS
 #include "fst_tc.cuh"
 
@@ -365,6 +366,14 @@ static fst_status set_attrs() {
   CU(cudaFuncSetAttribute(k_passB<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
   CU(cudaFuncSetAttribute(k_passC<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
   CU(cudaFuncSetAttribute(k_passC<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
+  CU(cudaFuncSetAttribute(k_sym_c<false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
+  CU(cudaFuncSetAttribute(k_sym_c<false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
+  CU(cudaFuncSetAttribute(k_sym_c<false, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
+  CU(cudaFuncSetAttribute(k_sym_c<true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
+  CU(cudaFuncSetAttribute(k_sym_c<true, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
+  CU(cudaFuncSetAttribute(k_sym_c<true, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
+  CU(cudaFuncSetAttribute(k_sym_z<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
+  CU(cudaFuncSetAttribute(k_sym_z<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
   CU(cudaFuncSetAttribute(k_coef_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
   CU(cudaFuncSetAttribute(k_expand_gemm<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
   CU(cudaFuncSetAttribute(k_expand_gemm<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
@@ -377,7 +386,6 @@ static fst_status set_attrs() {
   CU(cudaFuncSetAttribute(k_fastAw<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, fastw_smem(16)), "attr");
   CU(cudaFuncSetAttribute(k_fastAw<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, fastw_smem(8)), "attr");
   CU(cudaFuncSetAttribute(k_corr_cc, cudaFuncAttributeMaxDynamicSharedMemorySize, cc_smem(64)), "attr");
-  CU(cudaFuncSetAttribute(k_zadd, cudaFuncAttributeMaxDynamicSharedMemorySize, za_smem(64, 1)), "attr");
   CU(cudaFuncSetAttribute(k_fastB8192, cudaFuncAttributeMaxDynamicSharedMemorySize, fastb8192_smem()), "attr");
   CU(cudaFuncSetAttribute(k_fastB4096_2s, cudaFuncAttributeMaxDynamicSharedMemorySize, fastb2s_smem()), "attr");
   CU(cudaFuncSetAttribute(k_rcorr_part, cudaFuncAttributeMaxDynamicSharedMemorySize, rcorr_smem()), "attr");
@@ -976,30 +984,48 @@ struct DevRunner : Runner {
     LAUNCHED("k_rzadd");
     return FST_OK;
   }
+  // chunks of S_T^T y: about three blocks per SM in all (two are resident), at least a tile each, and
+  // no more partials than the scratch of the other forms holds (CORR_BLOCK samples each)
+  int sym_chunks(const ConvArgs<float> &a) override {
+    const int64_t rows = a.cplx ? 2 * a.batch : a.batch;
+    const int64_t groups = (rows + sy_rows(rows) - 1) / sy_rows(rows), tiles = ((a.N + 1) / 2 + SY_TN - 1) / SY_TN;
+    if (groups > 65535 || a.N < 4 * SY_TN) return 0;
+    const int64_t most = std::max<int64_t>((a.N + CORR_BLOCK - 1) / CORR_BLOCK, tc_slices(a.N));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(tiles, most), 3 * (int64_t)sms / groups));
+  }
+  fst_status sym_c(const ConvArgs<float> &a) override {
+    TRY(set_attrs());
+    const int64_t rows = a.cplx ? 2 * a.batch : a.batch;
+    const int RB = sy_rows(rows);
+    dim3 grid((unsigned)a.nkb, (unsigned)((rows + RB - 1) / RB));
+    const size_t smem = sy_smem(a.ncord, a.r - a.ncord, RB);
+    auto go = [&](auto kernel) { PROF("k_sym_c", a.npairs, (kernel<<<grid, 256, smem, cur>>>(a, a.cord, a.ncord, a.nkb))); };
+    if (a.cplx) go(RB == 8 ? k_sym_c<true, 8> : RB == 16 ? k_sym_c<true, 16> : k_sym_c<true, 32>);
+    else go(RB == 8 ? k_sym_c<false, 8> : RB == 16 ? k_sym_c<false, 16> : k_sym_c<false, 32>);
+    LAUNCHED("k_sym_c");
+    return FST_OK;
+  }
+  fst_status sym_z(const ConvArgs<float> &a) override {
+    TRY(set_attrs());
+    const int64_t rows = a.cplx ? 2 * a.batch : a.batch, H = (a.N + 1) / 2;
+    const int ng = sy_ng(rows);
+    const int64_t rg = (rows + SY_R * ng - 1) / (SY_R * ng);
+    // blocks of 64 threads where those of 256 would leave SMs idle (one row of N = 70001: 35 blocks)
+    const int thr = (H * ng + 1023) / 1024 * rg < sms ? 64 : 256, ns = thr / ng;
+    if (rg > 65535) return fail(FST_EINVAL, "batch too large for the correction pass");
+    dim3 grid((unsigned)((H + 4 * ns - 1) / (4 * ns)), (unsigned)rg);
+    const size_t smem = (size_t)a.r * (SY_R * ng + 1) * sizeof(float);
+    const bool vec = a.N % 4 == 0 && ((uintptr_t)a.out % 16) == 0 && (a.ld * (a.cplx ? 8 : 4)) % 16 == 0;
+    if (vec) PROF("k_sym_z", a.npairs, (k_sym_z<true><<<grid, thr, smem, cur>>>(a, a.cord, a.ncord)));
+    else PROF("k_sym_z", a.npairs, (k_sym_z<false><<<grid, thr, smem, cur>>>(a, a.cord, a.ncord)));
+    LAUNCHED("k_sym_z");
+    return FST_OK;
+  }
   fst_status corr_cc(const ConvArgs<float> &a) override {
     TRY(set_attrs());
     PROF("k_corr_cc", a.npairs,
          (k_corr_cc<<<(unsigned)((a.N + CORR_BLOCK - 1) / CORR_BLOCK), CC_THREADS, cc_smem(a.rpad), cur>>>(a)));
     LAUNCHED("k_corr_cc");
-    return FST_OK;
-  }
-  fst_status zadd(const ConvArgs<float> &a) override {
-    TRY(set_attrs());
-    const int64_t rows = a.cplx ? 2 * a.batch : a.batch;
-    const int ng = za_groups(rows), ns = ZA_THREADS / ng;
-    const int64_t nrb = (rows + ng * ZA_RG - 1) / (ng * ZA_RG);
-    const int64_t blocks = nrb * ((a.N + ns - 1) / ns);
-    if (blocks >= (1LL << 31)) return fail(FST_EINVAL, "batch too large for the correction pass");
-    PROF("k_zadd", a.npairs, (k_zadd<<<(unsigned)blocks, ZA_THREADS, za_smem(a.rpad, ng), cur>>>(a)));
-    LAUNCHED("k_zadd");
-    return FST_OK;
-  }
-  fst_status z_rmw(const ConvArgs<float> &a, const float *ST) override {
-    const int nsig = a.cplx ? ZR_ROWS / 2 : ZR_ROWS;
-    dim3 grid((unsigned)((a.N + ZR_N - 1) / ZR_N), (unsigned)((a.batch + nsig - 1) / nsig));
-    if (a.rpad <= 32) PROF("k_z_rmw", a.npairs, (k_z_rmw<32><<<grid, ZR_THREADS, 0, cur>>>(a, ST)));
-    else PROF("k_z_rmw", a.npairs, (k_z_rmw<64><<<grid, ZR_THREADS, 0, cur>>>(a, ST)));
-    LAUNCHED("k_z_rmw");
     return FST_OK;
   }
   fst_status corr_reduce(const ConvArgs<float> &a, const float *scale) override {

@@ -938,165 +938,6 @@ __global__ void k_corr_reduce(const ConvArgs<float> a, const float *scale) {
 }
 
 // ---------------------------------------------------------------------------
-// out += S_T a for every signal (the last step of the separate correction, a = D o S_T^T y
-// already summed): r <= RMAX FP32 FMAs per output value, on CUDA cores.
-// A block takes ZR_N consecutive samples and ZR_ROWS rows of a (real signals, or the (re, im)
-// rows of ZR_ROWS / 2 complex signals).  The S_T rows of its samples are contiguous in memory:
-// staged through shared memory with coalesced loads, then each thread keeps the row of its
-// sample in registers and walks half of the a rows (read as shared-memory broadcasts),
-// adding into out.  grid (ceil(N / ZR_N), ceil(rows / ZR_ROWS)), ZR_THREADS threads.
-// ---------------------------------------------------------------------------
-template <int RMAX>
-__global__ void __launch_bounds__(ZR_THREADS) k_z_rmw(const ConvArgs<float> a, const float *ST) {
-  __shared__ float st[ZR_N][RMAX + 1];
-  __shared__ float as[ZR_ROWS][RMAX];
-  const int r = a.r;
-  const int64_t n0 = (int64_t)blockIdx.x * ZR_N;
-  const int nsig = a.cplx ? ZR_ROWS / 2 : ZR_ROWS;
-  const int64_t sig0 = (int64_t)blockIdx.y * nsig;
-  // S_T rows n0 .. n0 + ZR_N - 1: ZR_N x rpad contiguous floats (rpad <= RMAX)
-  const int64_t nn = (a.N - n0 < ZR_N) ? a.N - n0 : ZR_N;
-  for (int t = threadIdx.x; t < ZR_N * a.rpad; t += ZR_THREADS) {
-    const int row = t / a.rpad, j = t % a.rpad;
-    st[row][j] = (row < nn && j < r) ? __ldg(ST + n0 * a.rpad + t) : 0.f;
-  }
-  for (int t = threadIdx.x; t < ZR_N * (RMAX - a.rpad); t += ZR_THREADS) {
-    const int row = t / (RMAX - a.rpad), j = a.rpad + t % (RMAX - a.rpad);
-    st[row][j] = 0.f;
-  }
-  // a rows: real signal sig0 + rr; complex signal sig0 + rr / 2, part rr & 1.  The rows of
-  // acoef are (pair 2 + part); for real signals that index is the signal itself.
-  for (int t = threadIdx.x; t < ZR_ROWS * RMAX; t += ZR_THREADS) {
-    const int rr = t / RMAX, j = t % RMAX;
-    const int64_t sg = a.cplx ? sig0 + rr / 2 : sig0 + rr;
-    const int64_t arow = a.cplx ? 2 * sg + (rr & 1) : sg;
-    as[rr][j] = (sg < a.batch && j < r) ? a.acoef[arow * a.rpad + j] : 0.f;
-  }
-  __syncthreads();
-  const int i = threadIdx.x % ZR_N, half = threadIdx.x / ZR_N;
-  const int64_t n = n0 + i;
-  if (n >= a.N) return;
-  float sv[RMAX];
-#pragma unroll
-  for (int j = 0; j < RMAX; ++j) sv[j] = st[i][j];
-  if (!a.cplx) {
-    const int rows = (int)(a.batch - sig0 < ZR_ROWS ? a.batch - sig0 : ZR_ROWS);
-    for (int rr = half; rr < rows; rr += 2) {
-      float z = 0.f;
-#pragma unroll
-      for (int j = 0; j < RMAX; ++j) z = fmaf(sv[j], as[rr][j], z);
-      a.out[(sig0 + rr) * a.ld + n] += z;
-    }
-  } else {
-    const int sigs = (int)(a.batch - sig0 < ZR_ROWS / 2 ? a.batch - sig0 : ZR_ROWS / 2);
-    for (int q = half; q < sigs; q += 2) {
-      float zr = 0.f, zi = 0.f;
-#pragma unroll
-      for (int j = 0; j < RMAX; ++j) {
-        zr = fmaf(sv[j], as[2 * q][j], zr);
-        zi = fmaf(sv[j], as[2 * q + 1][j], zi);
-      }
-      float2 *o = reinterpret_cast<float2 *>(a.out) + (sig0 + q) * a.ld + n;
-      float2 v = *o;
-      v.x += zr;
-      v.y += zi;
-      *o = v;
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
-// out += S_T a over the whole batch on CUDA cores (rpad <= 64): a block of ZA_THREADS threads
-// takes ns = ZA_THREADS / ng samples and up to 16 ng signal rows (ng = ceil(rows / 16), at
-// most 8: real signals, or the (re, im) rows of complex ones; row b of a is acoef row b).  The
-// block's S_T rows are staged once in shared memory, [sample][j] with a 16-byte aligned odd
-// stride (conflict-free float4 reads), and its a rows transposed to [j][row] (float4
-// broadcasts).  Thread (sample i, row group g) keeps ZA_RG sums in registers: per 4 j, one
-// float4 of S and ZA_RG / 4 float4 of a feed 4 ZA_RG FMAs.  Then the sums are added into out
-// (coalesced along the samples).
-// 1-D grid of ceil(N / ns) x (row blocks) blocks, block b = sample block b / nrb, row block
-// b % nrb: the row blocks of the same samples run side by side, so their S_T rows come from L2.
-// ---------------------------------------------------------------------------
-constexpr int ZA_THREADS = 256, ZA_RG = 16, ZA_ROWS = 128;
-// row groups per block: ceil(rows / 16) rounded up to a power of two, at most 8, so that
-// ZA_THREADS / ng samples times ng groups is exactly the block
-__host__ __device__ inline int za_groups(int64_t rows) {
-  int g = 1;
-  while (g < ZA_ROWS / ZA_RG && (int64_t)g * ZA_RG < rows) g *= 2;
-  return g;
-}
-__host__ __device__ inline int za_smem(int rpad, int ng) {
-  return ((ZA_THREADS / ng) * (rpad + 4) + rpad * (ng * ZA_RG + 4)) * 4;
-}
-
-__global__ void __launch_bounds__(ZA_THREADS) k_zadd(const ConvArgs<float> a) {
-  extern __shared__ __align__(16) float zsm[];
-  const int rpad = a.rpad, sst = rpad + 4;
-  const int64_t rows = a.cplx ? 2 * a.batch : a.batch;
-  const int ng = za_groups(rows), ns = ZA_THREADS / ng, brows = ng * ZA_RG, ast = brows + 4;
-  float *st = zsm;                        // [ns][sst]
-  float *as = zsm + ns * sst;             // [rpad][ast]
-  const int64_t nrb = (rows + brows - 1) / brows;
-  const int64_t row0 = ((int64_t)blockIdx.x % nrb) * brows;
-  const int nrow = (int)(rows - row0 < brows ? rows - row0 : brows);
-  const int64_t n0 = ((int64_t)blockIdx.x / nrb) * ns;
-  // S_T rows n0 .. n0 + ns - 1 (zero past N)
-  for (int e = threadIdx.x; e < ns * (rpad / 4); e += ZA_THREADS) {
-    const int i = e / (rpad / 4), q = e % (rpad / 4);
-    float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (n0 + i < a.N) v = __ldg(reinterpret_cast<const float4 *>(a.ST + (n0 + i) * rpad) + q);
-    *reinterpret_cast<float4 *>(st + i * sst + 4 * q) = v;
-  }
-  // a rows of this block, transposed: as[j][row]
-  for (int e = threadIdx.x; e < rpad * brows; e += ZA_THREADS) {
-    const int rr = e / rpad, j = e % rpad;
-    as[j * ast + rr] = (rr < nrow && j < a.r) ? a.acoef[(row0 + rr) * rpad + j] : 0.f;
-  }
-  __syncthreads();
-  const int i = threadIdx.x % ns, g = threadIdx.x / ns;
-  const int64_t n = n0 + i;
-  float acc[ZA_RG];
-#pragma unroll
-  for (int q = 0; q < ZA_RG; ++q) acc[q] = 0.f;
-  const float *srow = st + i * sst;
-  const float *acol = as + g * ZA_RG;
-  for (int j = 0; j < rpad; j += 4) {
-    const float4 s4 = *reinterpret_cast<const float4 *>(srow + j);
-#pragma unroll
-    for (int q = 0; q < ZA_RG; q += 4) {
-      const float4 a0 = *reinterpret_cast<const float4 *>(acol + (j + 0) * ast + q);
-      const float4 a1 = *reinterpret_cast<const float4 *>(acol + (j + 1) * ast + q);
-      const float4 a2 = *reinterpret_cast<const float4 *>(acol + (j + 2) * ast + q);
-      const float4 a3 = *reinterpret_cast<const float4 *>(acol + (j + 3) * ast + q);
-      acc[q + 0] = fmaf(s4.w, a3.x, fmaf(s4.z, a2.x, fmaf(s4.y, a1.x, fmaf(s4.x, a0.x, acc[q + 0]))));
-      acc[q + 1] = fmaf(s4.w, a3.y, fmaf(s4.z, a2.y, fmaf(s4.y, a1.y, fmaf(s4.x, a0.y, acc[q + 1]))));
-      acc[q + 2] = fmaf(s4.w, a3.z, fmaf(s4.z, a2.z, fmaf(s4.y, a1.z, fmaf(s4.x, a0.z, acc[q + 2]))));
-      acc[q + 3] = fmaf(s4.w, a3.w, fmaf(s4.z, a2.w, fmaf(s4.y, a1.w, fmaf(s4.x, a0.w, acc[q + 3]))));
-    }
-  }
-  if (n >= a.N) return;
-  if (!a.cplx) {
-#pragma unroll
-    for (int q = 0; q < ZA_RG; ++q) {
-      const int rr = g * ZA_RG + q;
-      if (rr < nrow) a.out[(row0 + rr) * a.ld + n] += acc[q];
-    }
-  } else {
-#pragma unroll
-    for (int q = 0; q < ZA_RG; q += 2) {
-      const int rr = g * ZA_RG + q;
-      if (rr < nrow) {
-        float2 *o = reinterpret_cast<float2 *>(a.out) + ((row0 + rr) >> 1) * a.ld + n;
-        float2 v = *o;
-        v.x += acc[q];
-        v.y += acc[q + 1];
-        *o = v;
-      }
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------
 // S_T^T y for small batches (at most CC_ROWS signal rows: real signals, or the (re, im) rows
 // of complex ones) on CUDA cores, in FP32: the MMA tile of the tensor-core kernel would be
 // mostly empty there and each k-tile's fixed cost dominates.  A block takes CORR_BLOCK

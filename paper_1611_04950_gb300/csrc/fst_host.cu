@@ -164,7 +164,17 @@ static bool tc_usable(const ConvArgs<float> &a) {
 static fst_status corr_coefficients(Runner *R, ConvArgs<float> &sc, const float *scale) {
   const int64_t rows = sc.cplx ? 2 * sc.batch : sc.batch;
   const int combos = (int)((rows + 3) / 4) * (sc.rpad / 8);
-  if (R->device() && sc.ST && rows <= 32 && sc.rpad <= 64 && combos <= 256 && (uintptr_t)sc.ST % 16 == 0 &&
+  // folded form on CUDA cores (half of S_T and of the FMAs) where the plan has the K-major S_T^T,
+  // except batches of more than 32 rows that the tcgen05 kernel can address at P <= 32: there it is
+  // the faster one beside the column passes (us for the whole call at N = 65536, r = 22, folded /
+  // tcgen05: 32 rows 41 / 62, 64 rows 76 / 73, 512 rows 433 / 394; two-stage lengths: 64 complex
+  // signals of 2^18 518 / 541, 64 real ones of 2^20 1050 / 1152)
+  const bool tc_better = rows > 32 && sc.N <= 65536 && tc_usable(sc);
+  const int sym = R->device() && sc.STt && sc.cord && !plain_mode() && !tc_better ? R->sym_chunks(sc) : 0;
+  if (sym > 0) {
+    sc.nkb = sym;
+    TRY(R->sym_c(sc));
+  } else if (R->device() && sc.ST && rows <= 32 && sc.rpad <= 64 && combos <= 256 && (uintptr_t)sc.ST % 16 == 0 &&
       !plain_mode()) {
     // few signal rows: FP32 CUDA-core partials (the tensor-core tile would be mostly empty)
     sc.nkb = (int)((sc.N + CORR_BLOCK - 1) / CORR_BLOCK);
@@ -193,12 +203,16 @@ static fst_status run_conv(Runner *R, const Layout &L, ConvArgs<T> a, int64_t np
   const int lanes = R->lanes();
   const size_t slot = slot_bytes(L, sizeof(T) == 8, a.rpad, a.mode == MODE_FORWARD);
   // separate correction (FP32 device): a = D o S_T^T y over every pair first (before any
-  // output is written, so y == out works); on tcgen05 whenever the signal rows allow a
-  // tensor map, else (P > 32) mma.sync kernels.  Then out += S_T a: in the fast column
-  // pass C, or by a last kernel over the whole batch.
+  // output is written, so y == out works).  Then out += S_T a: in the fast column pass C, or by
+  // a last kernel over the whole batch.
   const bool want = a.mode == MODE_FULL && a.r > 0 && sizeof(T) == 4 && R->device() && !L.small;
   const bool tc = want && tc_usable(*reinterpret_cast<const ConvArgs<float> *>(&a));
-  const bool split = want && (L.split_corr || tc);
+  const ConvArgs<float> &af = *reinterpret_cast<const ConvArgs<float> *>(&a);
+  // (at P = 8 and 17 to 64 rows no tensor map can address, the column pass's own products are the
+  // faster ones: 33 rows of 9001 samples 21.1 us, folded 23.6)
+  const int64_t nrows = a.cplx ? 2 * a.batch : a.batch;
+  const bool sym = af.STt && af.cord && !plain_mode() && !(L.fast && L.log2P == 3 && nrows > 16 && nrows <= 64);
+  const bool split = want && (L.split_corr || tc || sym);
   ConvArgs<float> sc{};
   if (split) {
     sc = *reinterpret_cast<const ConvArgs<float> *>(&a);
@@ -236,7 +250,7 @@ static fst_status run_conv(Runner *R, const Layout &L, ConvArgs<T> a, int64_t np
       TRY(R->passA(a, L));
       if (a.mode == MODE_FULL && a.r > 0 && !(L.fused_reduce && R->device())) TRY(R->reduce(a, L));
       TRY(R->passB(a, L));
-      if (split && L.fast && !waited[lane]) {
+      if (split && !waited[lane] && (L.fast || (const void *)a.y == (const void *)a.out)) {
         R->wait_side();
         waited[lane] = true;
       }
@@ -248,10 +262,8 @@ static fst_status run_conv(Runner *R, const Layout &L, ConvArgs<T> a, int64_t np
     // out += S_T a over the whole batch once both lanes have written B y
     R->lanes_join_first();
     R->wait_side();
-    // CUDA-core pass with register-blocked sums (any batch, rpad <= 64), else mma.sync
-    const bool za_ok = sc.ST && sc.rpad <= 64 && (!sc.cplx || (uintptr_t)sc.out % 8 == 0) &&
-                       (uintptr_t)sc.ST % 16 == 0;
-    if (za_ok) TRY(R->zadd(sc));
+    // folded CUDA-core pass (r <= 128), else mma.sync
+    if (sc.STt && sc.cord) TRY(R->sym_z(sc));
     else TRY(R->corr_z(sc));
   }
   return FST_OK;
@@ -377,6 +389,8 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
     a.STt = p->STt;
     a.tc_nB = p->tc_nB;
     a.tc_Npad = p->tc_Npad;
+    a.cord = p->cord;
+    a.ncord = p->ncord;
     a.twB = p->twB;
     a.tw8 = p->tw8;
     if (p->twS) {
@@ -963,6 +977,14 @@ static fst_status plan_end(fst_plan_t p, double *S, const std::vector<double> &l
     if ((s = R->alloc((void **)&p->STt, nt * sizeof(float))) != FST_OK) return bail(s);
     if ((s = R->tc_prep(p->ST32, N, (int)p->rpad, (int)p->r, p->tc_nB, p->tc_Npad, p->STt)) != FST_OK)
       return bail(s);
+    std::vector<int> ord;
+    for (int par = 0; par < 2; ++par) {
+      for (int64_t j = 0; j < p->r; ++j)
+        if ((p->idx[j] & 1) == par) ord.push_back((int)j);
+      if (par == 0) p->ncord = (int)ord.size();
+    }
+    if ((s = R->alloc((void **)&p->cord, ord.size() * sizeof(int))) != FST_OK) return bail(s);
+    if ((s = R->h2d(p->cord, ord.data(), ord.size() * sizeof(int))) != FST_OK) return bail(s);
     if ((s = R->sync()) != FST_OK) return bail(s);
   }
   if (R->device() && p->lay32.small && p->log2M >= 10 && p->rpad <= SM_RMAX) {
@@ -1055,6 +1077,7 @@ void destroy_plan(fst_plan_t p) {
     for (auto &e : p->graphs) R->graph_destroy(e.exec);
     p->graphs.clear();
     void *bufs[] = {p->spec32, p->ST32, p->D32, p->spec64, p->ST64, p->D64, p->ST32_hl, p->STt, p->spec_unit, p->cpar, p->twS, p->STs,
+                    p->cord,
                     p->tw32h, p->tw32l, p->tw64h, p->tw64l, p->twB, p->tw8, p->ws};
     for (void *b : bufs)
       if (b) R->release(b);
@@ -1469,6 +1492,8 @@ static fst_status coeffs_t(fst_plan_t p, const T *y, c2<T> *out, int64_t batch, 
     ca.STt = p->STt;
     ca.tc_nB = p->tc_nB;
     ca.tc_Npad = p->tc_Npad;
+    ca.cord = p->cord;
+    ca.ncord = p->ncord;
     const int64_t nK = std::max<int64_t>((N + CORR_BLOCK - 1) / CORR_BLOCK, tc_slices(N));
     ca.part = (float *)c.partU;
     ca.acoef = (float *)c.partU + (size_t)npairs * nK * 2 * p->rpad;

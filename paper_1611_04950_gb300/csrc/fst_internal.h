@@ -103,8 +103,6 @@ struct Runner {
   virtual fst_status exp_scatter(const ExpArgs<double> &a, int64_t nsig, double2 *Xs) = 0;
   virtual fst_status expand(const ExpArgs<float> &a, int64_t nsig) = 0;
   virtual fst_status expand(const ExpArgs<double> &a, int64_t nsig) = 0;
-  // out += S_T a on CUDA cores (FP32, r <= 64)
-  virtual fst_status z_rmw(const ConvArgs<float> &a, const float *ST) { return FST_EUNSUPPORTED; }
   // ragged four-step signals (FP32 device): correction partials per item, a per signal, and
   // out += S_T a per item (descriptor arrays in runner memory)
   virtual fst_status rcorr(const RSig *sigs, int nsig, const RItem *items, int nitems, int cplx, float *part,
@@ -114,8 +112,10 @@ struct Runner {
   }
   // S_T^T y partials per CORR_BLOCK samples on CUDA cores (FP32, at most 32 signal rows, rpad <= 64)
   virtual fst_status corr_cc(const ConvArgs<float> &a) { return FST_EUNSUPPORTED; }
-  // out += S_T a on CUDA cores over the whole batch (FP32, rpad <= 64, any number of rows)
-  virtual fst_status zadd(const ConvArgs<float> &a) { return FST_EUNSUPPORTED; }
+  // folded correction (fst_sym.cuh): chunks it wants, partials per chunk, out += S_T a
+  virtual int sym_chunks(const ConvArgs<float> &a) { return 0; }
+  virtual fst_status sym_c(const ConvArgs<float> &a) { return FST_EUNSUPPORTED; }
+  virtual fst_status sym_z(const ConvArgs<float> &a) { return FST_EUNSUPPORTED; }
 
   // plan kernels (all pointers in runner memory)
   // batched eigen-targets of one or many plans (descriptors and data in runner memory):
@@ -204,6 +204,8 @@ struct fst_plan_s {
   // stage twiddles of the 4096-point row FFT: [t][k] = W_256^{k t} (k < 16), then
   // W_4096^{k t} (k < 256), t < 16
   float2 *twB = nullptr;
+  int *cord = nullptr;     // columns of S_T, the ncord symmetric ones first (plans with STt)
+  int ncord = 0;
   float2 *twS = nullptr;   // single-CTA path: its stage twiddles (device plans, M = 2^10 .. 2^14), and
   float *STs = nullptr;    // the K-major copy of S_T, [r][N]
   float2 *tw8 = nullptr;   // stage twiddles of the 8192-point row FFT (FP64 built)

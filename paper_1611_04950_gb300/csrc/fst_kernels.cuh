@@ -37,8 +37,6 @@ enum { MODE_FULL = 0, MODE_CONV = 1, MODE_FORWARD = 2, MODE_ZONLY = 3 };
 
 constexpr int CORR_ROWS = 512;    // samples per tensor-core tile of the separate correction kernels
 constexpr int CORR_BLOCK = 2048;  // samples per partial sum of S_T^T y (four tiles)
-// CUDA-core out += S_T a: threads, samples and signal rows per block
-constexpr int ZR_THREADS = 256, ZR_N = 128, ZR_ROWS = 64;
 
 // Launch layout of the length-M transform for one real type.
 struct Layout {
@@ -137,6 +135,8 @@ template <typename T> struct ConvArgs {
   int64_t tc_Npad;
   const float2 *twB;  // FP32 device plans: stage twiddles of the 4096-point row FFT, then W_1024^t
   const float2 *tw8;  // FP32 device plans: stage twiddles of the 8192-point row FFT
+  const int *cord;    // FP32 device plans with STt: columns of S_T, the ncord symmetric ones first
+  int ncord;
   const float2 *twS;  // FP32 device plans of the single-CTA path: stage twiddles, S_T's antisymmetric
   unsigned odd[4];    // columns as bits (STt then holds its K-major copy, rows tc_Npad apart)
   const c2<T> *exp_c; // forward transform of T1 c: coefficient vectors, exp_kp apart, bins -exp_h..exp_h first

@@ -1,0 +1,38 @@
+"""The folded rank-r correction (fst_sym.cuh) at its edges: odd N (the middle sample), N with every
+remainder mod 4 (16-byte and single accesses), 1 to 130 rows (every block height and row-group count),
+strided and unaligned rows, complex signals, in place, ranks from one column tile to several.  Against
+the FP64 oracle; tolerance 1e-5 of ||y||, the FP32 tolerance of the parity tests."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+
+pytestmark = pytest.mark.gpu
+
+from paper_1611_04950_gb300 import fst as F  # noqa: E402
+from paper_1611_04950_gb300 import workloads  # noqa: E402
+from oracle import fst_oracle as O  # noqa: E402
+
+
+@pytest.mark.parametrize("N,W,eps", [(9001, 0.2, 1e-1), (10002, 0.1, 1e-6), (20003, 0.25, 1e-8), (66000, 0.05, 1e-6),
+                                     (70001, 0.2, 1e-12), (131074, 0.1, 1e-4)])
+@pytest.mark.parametrize("batch,cplx", [(1, False), (1, True), (5, True), (9, False), (17, True), (33, False), (65, True)])
+def test_folded_correction(N, W, eps, batch, cplx):
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    p = F.Plan(N, W, eps=eps)
+    o = O.make_plan(N, W, p.K, eps)
+    assert p.r == o.r
+    y = workloads.gaussian(batch, N, seed=N + batch, complex_=cplx).to(torch.complex64 if cplx else torch.float32)
+    nrm = np.linalg.norm(y.numpy(), axis=1)
+    pick = sorted({0, batch // 2, batch - 1})
+    ref = O.fast_project(o, y.numpy()[pick].astype(np.complex128 if cplx else np.float64).T).T
+    yd = y.to("cuda")
+    out = p.project(yd)
+    assert np.all(np.linalg.norm(out.cpu().numpy()[pick] - ref, axis=1) < 1e-5 * nrm[pick])
+    assert torch.equal(p.project(yd), out)
+    flat = torch.zeros(batch * (N + 3) + 1, dtype=y.dtype, device="cuda")
+    wide = flat[1:].view(batch, N + 3)[:, :N]            # odd stride and base
+    wide.copy_(yd)
+    got = p.project(wide, out=wide)                      # in place
+    assert np.all(np.linalg.norm(got.cpu().numpy()[pick] - ref, axis=1) < 1e-5 * nrm[pick])
