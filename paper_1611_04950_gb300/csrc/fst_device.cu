@@ -526,7 +526,42 @@ struct DevRunner : Runner {
       if (cap[i]) cudaStreamDestroy(cap[i]);
     for (cudaEvent_t e : {fork, join, ev_mid, ev_side, join_side, t0, t1})
       if (e) cudaEventDestroy(e);
+    for (cudaStream_t b : br)
+      if (b) cudaStreamDestroy(b);
+    for (cudaEvent_t e : br_ev)
+      if (e) cudaEventDestroy(e);
     if (tc_err_h) cudaFreeHost(tc_err_h);
+  }
+  static constexpr int BRANCHES = 6;
+  cudaStream_t br[BRANCHES] = {};
+  cudaEvent_t br_ev[BRANCHES + 1] = {};
+  bool br_on[BRANCHES] = {};
+  fst_status branch(int k) override {
+    cur = s;
+    if (k < 0) return FST_OK;
+    k %= BRANCHES;
+    if (!br[k]) {
+      CU(cudaStreamCreateWithFlags(&br[k], cudaStreamNonBlocking), "stream");
+      CU(cudaEventCreateWithFlags(&br_ev[k], cudaEventDisableTiming), "event");
+    }
+    if (!br_ev[BRANCHES]) CU(cudaEventCreateWithFlags(&br_ev[BRANCHES], cudaEventDisableTiming), "event");
+    if (!br_on[k]) {
+      CU(cudaEventRecord(br_ev[BRANCHES], s), "event");
+      CU(cudaStreamWaitEvent(br[k], br_ev[BRANCHES], 0), "wait");
+      br_on[k] = true;
+    }
+    cur = br[k];
+    return FST_OK;
+  }
+  fst_status branch_join() override {
+    cur = s;
+    for (int k = 0; k < BRANCHES; ++k)
+      if (br_on[k]) {
+        br_on[k] = false;
+        CU(cudaEventRecord(br_ev[k], br[k]), "event");
+        CU(cudaStreamWaitEvent(s, br_ev[k], 0), "wait");
+      }
+    return FST_OK;
   }
   cudaEvent_t t0 = nullptr, t1 = nullptr;
   fst_status timer(int phase, double *ms) override {
@@ -1588,7 +1623,10 @@ extern "C" fst_status fst_project_ragged(const fst_plan_t *plans, const void *co
   for (int64_t i = 0; i < count; ++i) plans[i]->R->set_stream((void *)g_ragged_cap);
   const long long l0 = g_launches;
   CU(cudaStreamBeginCapture(g_ragged_cap, cudaStreamCaptureModeThreadLocal), "cudaStreamBeginCapture");
+  ctx->state.branches = true;
   fst_status st = run_ragged(plans, y, out, count, dtype, ctx->state);
+  ctx->state.branches = false;
+  if (st != FST_OK) plans[0]->R->branch_join();   // no branch may be left in the capture
   cudaGraph_t g = nullptr;
   cudaError_t e = cudaStreamEndCapture(g_ragged_cap, &g);
   for (int64_t i = 0; i < count; ++i) plans[i]->R->set_stream(stream);

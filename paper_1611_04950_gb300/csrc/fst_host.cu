@@ -1811,13 +1811,18 @@ static bool autotune_enabled() {
 //      a time (re, im), each with its own data, length and spectrum (4096-point rows: the row
 //      pass applies both spectra; other row lengths: one real signal per slot);
 //   3. out_i += S_T,i a_i over all items (one launch).
+// While a batch is recorded (st.branches) 1. runs on a branch beside 2., whose classes share two
+// lanes, and so do the single-CTA signals; only 3. waits for all of it.  Signals in place keep the
+// order (1. reads what 2. overwrites).  256 signals of 1000 .. 262144 samples: 736 -> 563 us.
 // The pairs per launch group of each class are picked on the first call (autotuner: the
 // candidate groupings of 16 .. 256 MiB of intermediate are timed with device events and the
 // fastest kept; the grouping does not change the arithmetic, so results do not depend on it).
 static fst_status ragged_fourstep_f32(const fst_plan_t *plans, const void *const *y, void *const *out,
-                                      const std::vector<int64_t> &idx, bool cplx, RaggedState &st) {
-  Runner *R = plans[idx[0]]->R;
+                                      const std::vector<int64_t> &idx, bool cplx, RaggedState &st, Runner *R) {
   const int nsig = (int)idx.size();
+  bool inplace_any = false;
+  for (int64_t i : idx) inplace_any = inplace_any || y[i] == out[i];
+  const bool br = st.branches && !inplace_any;
   // correction descriptors and items
   std::vector<RSig> sig(nsig);
   std::vector<RItem> items;
@@ -1847,8 +1852,10 @@ static fst_status ragged_fourstep_f32(const fst_plan_t *plans, const void *const
                  &ditems));
   TRY(ragged_buf(R, st, (size_t)std::max<int64_t>(poff, 1) * sizeof(float), nullptr, &dpart));
   TRY(ragged_buf(R, st, (size_t)nsig * 2 * RC_RMAX * sizeof(float), nullptr, &dacoef));
+  if (br) TRY(R->branch(0));
   TRY(R->rcorr((const RSig *)dsig, nsig, (const RItem *)ditems, (int)items.size(), cplx ? 1 : 0, (float *)dpart,
                (float *)dacoef));
+  TRY(R->branch(-1));
 
   // length classes
   std::vector<std::vector<int>> cls(32);
@@ -1857,16 +1864,26 @@ static fst_status ragged_fourstep_f32(const fst_plan_t *plans, const void *const
     st.chunk.assign(32, 0);
     st.tune_ms.assign(32, 0.0);
   }
-  // one intermediate workspace for every class (they run one after the other): 256 MiB at most
+  // an intermediate workspace for each of two lanes of classes (256 MiB at most): a class goes to
+  // the lane with less work so far, longest first
   size_t ws_max = 0;
   for (int lg = 0; lg < 32; ++lg)
     if (!cls[lg].empty())
       ws_max = std::max(ws_max, std::min<size_t>((size_t)cls[lg].size(), std::max<size_t>(1, (256u << 20) >> (lg + 3))) *
                                     ((size_t)8 << lg));
-  void *dws;
-  TRY(ragged_buf(R, st, ws_max, nullptr, &dws));
-  for (int lg = 0; lg < 32; ++lg) {
-    if (cls[lg].empty()) continue;
+  void *dws[2];
+  double load[2] = {0.0, 0.0};
+  for (int k = 0; k < 2; ++k) TRY(ragged_buf(R, st, ws_max, nullptr, &dws[k]));
+  std::vector<int> order;
+  for (int lg = 0; lg < 32; ++lg)
+    if (!cls[lg].empty()) order.push_back(lg);
+  auto work = [&](int lg) { return (double)cls[lg].size() * (double)(1LL << lg); };
+  std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return work(p) > work(q); });
+  for (int lg : order) {
+    const int lane = load[1] < load[0] ? 1 : 0;
+    load[lane] += work(lg);
+    if (br && lane) TRY(R->branch(1));
+    else TRY(R->branch(-1));
     const std::vector<int> &c = cls[lg];
     const int64_t cnt = (int64_t)c.size();
     fst_plan_t p0 = plans[idx[c[0]]];
@@ -1915,7 +1932,7 @@ static fst_status ragged_fourstep_f32(const fst_plan_t *plans, const void *const
     a.tw = plan_tw<float>(p0);
     a.twB = p0->twB;
     a.tw8 = p0->tw8;
-    a.inter = (float2 *)dws;
+    a.inter = (float2 *)dws[lane];
     a.mode = MODE_CONV;
     auto run_groups = [&](int64_t chunk) -> fst_status {
       for (int64_t q0 = 0; q0 < nslot; q0 += chunk) {
@@ -1955,6 +1972,8 @@ static fst_status ragged_fourstep_f32(const fst_plan_t *plans, const void *const
     }
     TRY(run_groups(st.chunk[lg]));
   }
+  TRY(R->branch(-1));
+  if (br) TRY(R->branch_join());
   return R->rzadd((const RSig *)dsig, (const RItem *)ditems, (int)items.size(), cplx ? 1 : 0, (const float *)dacoef);
 }
 
@@ -1963,6 +1982,8 @@ static fst_status ragged_t(const fst_plan_t *plans, const void *const *y, void *
                            bool cplx, RaggedState &st) {
   const bool dbl = sizeof(T) == 8;
   st.next = 0;
+  Runner *R0 = plans[0]->R;   // every launch that may go to a branch
+  int nbr = 0;
   // single-CTA signals by FFT length, one launch each
   std::vector<std::vector<RaggedDesc<T>>> buckets(32);
   std::vector<int> maxr(32, 0);
@@ -2016,7 +2037,10 @@ static fst_status ragged_t(const fst_plan_t *plans, const void *const *y, void *
     }
     if (sd.size() == buckets[lg].size()) {
       TRY(ragged_buf(R, st, sd.size() * sizeof(SmallDesc), sd.data(), &dd));
-      TRY(R->small32_ragged((const SmallDesc *)dd, (int)sd.size(), lg, maxr[lg], p0->twB, cplx ? 1 : 0));
+      // the lengths do not depend on each other, nor on the four-step signals
+      if (st.branches) TRY(R0->branch(2 + nbr++ % 4));
+      TRY(R0->small32_ragged((const SmallDesc *)dd, (int)sd.size(), lg, maxr[lg], p0->twB, cplx ? 1 : 0));
+      TRY(R0->branch(-1));
       continue;
     }
     TRY(ragged_buf(R, st, buckets[lg].size() * sizeof(RaggedDesc<T>), buckets[lg].data(), &dd));
@@ -2030,7 +2054,7 @@ static fst_status ragged_t(const fst_plan_t *plans, const void *const *y, void *
     base.npairs = 1;
     TRY(R->small_ragged((const RaggedDesc<T> *)dd, (int)buckets[lg].size(), base, L));
   }
-  if (others.empty()) return FST_OK;
+  if (others.empty()) return R0->branch_join();
   // FP32 device plans: batched four-step path; otherwise one call per signal
   bool batched = !dbl;
   for (int64_t i : others) {
@@ -2039,7 +2063,11 @@ static fst_status ragged_t(const fst_plan_t *plans, const void *const *y, void *
               (p->lay32.fast || p->lay32.big) && (!cplx || (uintptr_t)out[i] % 8 == 0) &&
               (!cplx || (uintptr_t)y[i] % 8 == 0);
   }
-  if (batched) return ragged_fourstep_f32(plans, y, out, others, cplx, st);
+  if (batched) {
+    TRY(ragged_fourstep_f32(plans, y, out, others, cplx, st, R0));
+    return R0->branch_join();
+  }
+  TRY(R0->branch_join());
   for (int64_t i : others)
     TRY(run_apply(plans[i], y[i], out[i], 1, 0, cplx ? (dbl ? FST_C128 : FST_C64) : (dbl ? FST_F64 : FST_F32), true));
   return FST_OK;

@@ -45,6 +45,11 @@ struct Runner {
   virtual void use_side() {}
   virtual void side_done() {}
   virtual void wait_side() {}
+  // branches of a recorded ragged batch (device runner): branch(k) orders side stream k after what
+  // the base stream has issued at its first use since the last branch_join(), and makes it current;
+  // branch(-1) returns to the base stream; branch_join() orders the base stream after all of them
+  virtual fst_status branch(int) { return FST_OK; }
+  virtual fst_status branch_join() { return FST_OK; }
   virtual fst_status alloc(void **p, size_t bytes) = 0;
   virtual void release(void *p) = 0;
   virtual fst_status h2d(void *dst, const void *src, size_t bytes) = 0;
@@ -245,6 +250,7 @@ bool profiling_enabled();   // per-launch event timing is on (fst_profile_enable
 // Device buffers and launch choices of one ragged signature (owned by the caller): the first
 // call allocates in a fixed order, later calls with the same signature reuse them in that order
 struct RaggedState {
+  bool branches = false;            // recording: independent parts of the batch go to branches
   std::vector<void *> bufs;
   size_t next = 0;                  // cursor into bufs during a call
   bool tuned = false;
