@@ -1160,14 +1160,14 @@ struct DevRunner : Runner {
     LAUNCHED("k_coef_lowrank");
     return FST_OK;
   }
-  // one block per half SM (two fit) over the vector groups; 113 KB of shared memory at most
+  // one block per SM over the vector groups; two tile buffers in shared memory
   int lowrank_plan(int64_t N, int rH, int DA, int DB, int64_t nvc, size_t *scratch) override {
     const int64_t groups = (nvc + LR_VC - 1) / LR_VC, tiles = N / 2 / LR_TN;
     const LrShape sh = lr_shape(rH, DA, DB, (int)std::min<int64_t>(nvc, LR_VC));
     const LrShape s1 = lr_shape(rH, DA, DB, 1);
-    if (N < 2 * LR_TN || groups > 65535 || sh.kg < 1 || s1.kg < 1 || std::max(lr_smem(sh), lr_smem(s1)) > 113 * 1024)
+    if (N < 2 * LR_TN || groups > 65535 || sh.kg < 1 || s1.kg < 1 || std::max(lr_smem(sh), lr_smem(s1)) > 227 * 1024)
       return 0;
-    const int64_t n = std::max<int64_t>(1, std::min<int64_t>(tiles, 2 * (int64_t)sms / groups));
+    const int64_t n = std::max<int64_t>(1, std::min<int64_t>(tiles, (int64_t)sms / groups));
     *scratch = (size_t)(n * groups) * 64 * 256 * sizeof(float) + 256;
     return (int)n;
   }
@@ -1178,7 +1178,7 @@ struct DevRunner : Runner {
     for (int v : {(int)std::min<int64_t>(nvc, LR_VC), (int)(nvc % LR_VC)})
       if (v > 0) smem = std::max(smem, lr_smem(lr_shape(a.rH, a.DA, a.DB, v)));
     dim3 grid((unsigned)a.nchunks, (unsigned)((nvc + LR_VC - 1) / LR_VC));
-    PROF("k_coef_gemm", 0, (k_coef_gemm<<<grid, 256, smem, cur>>>(a, a.nchunks, (float *)scratch)));
+    PROF("k_coef_gemm", 0, (k_coef_gemm<<<grid, 512, smem, cur>>>(a, a.nchunks, (float *)scratch)));
     LAUNCHED("k_coef_gemm");
     return FST_OK;
   }

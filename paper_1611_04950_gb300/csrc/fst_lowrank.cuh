@@ -44,7 +44,7 @@ __host__ __device__ inline LrShape lr_shape(int rH, int DA, int DB, int vc) {
   return s;
 }
 __host__ __device__ inline size_t lr_smem(const LrShape &s) {
-  const size_t tile = (size_t)LR_TN * (s.cs + 4 * LR_VS), sums = (size_t)s.kg * s.ntile * 64;
+  const size_t tile = 2 * (size_t)LR_TN * (s.cs + 4 * LR_VS), sums = (size_t)s.kg * s.ntile * 64;
   return (tile > sums ? tile : sums) * 4;
 }
 
@@ -57,32 +57,44 @@ __device__ __forceinline__ float lr_zstep(const float *zfirst, const float *zshi
 }
 
 // ---------------------------------------------------------------------------
-// raw low-rank sums of T2^* y, grid (nchunk, vector groups), 256 threads, dynamic lr_smem
-//   a tile: 64 folded samples.  Threads 0-127 generate the Z columns (one of the two mirror
-//   samples each, combined by a shuffle), 128-255 the powers and the folded, phase-rotated
-//   vectors; then thread (column tile, vector tile, sample group) accumulates 8 x 8 sums: per
-//   sample 4 16-byte loads feed 32 packed FMAs.  Every LR_FLUSH tiles the sums are added to the
+// raw low-rank sums of T2^* y, grid (nchunk, vector groups), 512 threads, dynamic lr_smem
+//   a tile: 64 folded samples, two buffers.  The upper eight warps generate the next tile: four the
+//   Z columns (one of the two mirror samples a thread, combined by a shuffle), four the powers and
+//   the folded, phase-rotated vectors.  Meanwhile thread (column tile, vector tile, sample group)
+//   of the lower eight accumulates 8 x 8 sums of the current one: per sample 4 16-byte loads feed
+//   32 packed FMAs.  Named barriers 1, 2 (tile ready) and 3, 4 (buffer free) hand the buffers
+//   over: each side arrives exactly as often as the other waits.  Every LR_FLUSH tiles the sums are added to the
 //   block's own area of `scr`, which keeps the FP32 chains short; sample groups are added in order
 //   at the end.  Same output layout as coef_lowrank_body.
-// Measured, 16 real signals of N = 2^22, 38 + 38 + 31 columns: 3476 -> 919 us.
+// Measured, 16 real signals of N = 2^22, 38 + 38 + 31 columns: 3476 -> 770 us
+// (960 with all warps generating, then multiplying).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256, 2) k_coef_gemm(const CoefArgs<float> a, int nchunk, float *scr) {
+// half of a named barrier of all 512 threads: wait for it, or only count towards it
+__device__ __forceinline__ void lr_bar_sync(int id) {
+  __syncwarp();
+  asm volatile("bar.sync %0, 512;" ::"r"(id) : "memory");
+}
+__device__ __forceinline__ void lr_bar_arrive(int id) {
+  __syncwarp();
+  asm volatile("bar.arrive %0, 512;" ::"r"(id) : "memory");
+}
+__global__ void __launch_bounds__(512, 1) k_coef_gemm(const CoefArgs<float> a, int nchunk, float *scr) {
   extern __shared__ __align__(16) float lsm[];
   const int tid = threadIdx.x;
   const int64_t H = a.N / 2, nvc = a.cplx ? 2 * a.batch : a.batch;
   const int64_t c0 = (int64_t)blockIdx.y * LR_VC;
   const int vc = (int)(nvc - c0 < LR_VC ? nvc - c0 : LR_VC);
   const LrShape S = lr_shape(a.rH, a.DA, a.DB, vc);
-  float *cols = lsm, *V = lsm + LR_TN * S.cs;       // V: PA, DA, PB, DB, each [LR_TN][LR_VS]
+  const int tile_f = LR_TN * (S.cs + 4 * LR_VS);   // floats of a buffer: columns, then PA, DA, PB, DB, each [LR_TN][LR_VS]
   const int64_t ntl = (H + LR_TN - 1) / LR_TN;
   const int64_t t0 = ntl * blockIdx.x / nchunk, t1 = ntl * (blockIdx.x + 1) / nchunk;
   // this thread's sums
   const int id = tid % S.ntile, kgi = tid / S.ntile, vt = id % S.nvt, ct = id / S.nvt;
-  const bool on = kgi < S.kg;
+  const bool gen = tid >= 256, on = !gen && kgi < S.kg;
   const int ne = (S.nz + S.npe) / 8, nA = ne + (S.nz + S.npo) / 8;
   const int cA = ct < nA ? ct * 8 : (ct - nA < S.npe / 8 ? S.nz + (ct - nA) * 8 : 2 * S.nz + S.npe + (ct - nA - S.npe / 8) * 8);
   const int vsel = ct < nA ? (ct < ne ? 0 : 1) : (ct - nA < S.npe / 8 ? 2 : 3);
-  const float *cp = cols + cA, *vp = V + vsel * LR_TN * LR_VS + vt * 8;
+  const float *cp = lsm + cA, *vp = lsm + LR_TN * S.cs + vsel * LR_TN * LR_VS + vt * 8;
   float2 acc[8][4];
 #pragma unroll
   for (int i = 0; i < 8; ++i)
@@ -105,93 +117,117 @@ __global__ void __launch_bounds__(256, 2) k_coef_gemm(const CoefArgs<float> a, i
   const float Nd = (float)a.N, cen = (float)(0.5 * (double)(a.N - 1)), invN = (float)(1.0 / (double)a.N);
   int since = 0;
   for (int64_t t = t0; t < t1; ++t) {
-    const int64_t n0 = t * LR_TN;
-    __syncthreads();
-    if (tid < 128) {
-      const int i = tid >> 1, side = tid & 1;
-      const int64_t n = n0 + i;
-      const float xf = (float)n + 0.5f, x = side ? Nd - xf : xf;
-      float *dst = cols + i * S.cs + (side ? S.nz + S.npe : 0);
-      float z = __fdividef(a.zfirst[0], x + a.zshift[0]);
-      for (int k0 = 0; k0 < S.nz; k0 += 4) {
-        float v[4];
-#pragma unroll
-        for (int kk = 0; kk < 4; ++kk) {
-          const int k = k0 + kk;
-          if (k > 0 && k < a.rH) z *= lr_zstep(a.zfirst, a.zshift, k, x);
-          const float other = __shfl_xor_sync(0xffffffffu, z, 1);
-          v[kk] = k < a.rH ? (side ? other - z : z + other) : 0.f;
-        }
-        *reinterpret_cast<float4 *>(dst + k0) = make_float4(v[0], v[1], v[2], v[3]);
-      }
-    } else {
-      const int i = (tid - 128) & 63, g = (tid - 128) >> 6;
-      const int64_t n = n0 + i, m = a.N - 1 - n;
-      const float u = ((float)n - cen) * invN, u2 = u * u;
-      {
-        float p = g ? u : 1.f;
-        const int np = g ? S.npo : S.npe, D = (a.DA > a.DB ? a.DA : a.DB) - g;
-        float *dst = cols + i * S.cs + (g ? 2 * S.nz + S.npe : S.nz);
-        for (int k0 = 0; k0 < np; k0 += 4) {
+    const int buf = (int)((t - t0) & 1);
+    if (gen) {
+      if (t >= t0 + 2) lr_bar_sync(3 + buf);
+      float *cols = lsm + buf * tile_f, *V = cols + LR_TN * S.cs;
+      const int64_t n0 = t * LR_TN;
+      if (tid < 384) {
+        const int i = (tid - 256) >> 1, side = tid & 1;
+        const int64_t n = n0 + i;
+        const float xf = (float)n + 0.5f, x = side ? Nd - xf : xf;
+        float *dst = cols + i * S.cs + (side ? S.nz + S.npe : 0);
+        float z = __fdividef(a.zfirst[0], x + a.zshift[0]);
+        for (int k0 = 0; k0 < S.nz; k0 += 4) {
           float v[4];
 #pragma unroll
           for (int kk = 0; kk < 4; ++kk) {
-            v[kk] = 2 * (k0 + kk) < D ? p : 0.f;
-            p *= u2;
+            const int k = k0 + kk;
+            if (k > 0 && k < a.rH) z *= lr_zstep(a.zfirst, a.zshift, k, x);
+            const float other = __shfl_xor_sync(0xffffffffu, z, 1);
+            v[kk] = k < a.rH ? (side ? other - z : z + other) : 0.f;
           }
           *reinterpret_cast<float4 *>(dst + k0) = make_float4(v[0], v[1], v[2], v[3]);
         }
-      }
-      const bool in = n < H;
-      const float2 z2 = make_float2(0.f, 0.f);
-      const float2 pa = in ? a.phA[n] : z2, pam = in ? a.phA[m] : z2, pb = in ? a.phB[n] : z2, pbm = in ? a.phB[m] : z2;
-      for (int s = g; s < 4 * S.nvt; s += 2) {
-        float2 an = z2, am = z2, bn = z2, bm = z2;
-        if (in && s < vc) {
-          if (!a.cplx) {
-            const float *row = a.y + (c0 + s) * a.ld;
-            const float y1 = row[n], y2 = row[m];
-            an = cscale(pa, y1);
-            am = cscale(pam, y2);
-            bn = cscale(pb, y1);
-            bm = cscale(pbm, y2);
-          } else {
-            const float2 *row = reinterpret_cast<const float2 *>(a.y) + ((c0 + s) >> 1) * a.ld;
-            const float2 y1 = row[n], y2 = row[m];
-            const bool cj = ((c0 + s) & 1) != 0;
-            an = cmul(cj ? cconj(pa) : pa, y1);
-            am = cmul(cj ? cconj(pam) : pam, y2);
-            bn = cmul(cj ? cconj(pb) : pb, y1);
-            bm = cmul(cj ? cconj(pbm) : pbm, y2);
+      } else {
+        const int i = (tid - 384) & 63, g = (tid - 384) >> 6;
+        const int64_t n = n0 + i, m = a.N - 1 - n;
+        const bool in = n < H;
+        const float2 z2 = make_float2(0.f, 0.f);
+        // every load of the tile first: signals s = g + 2 q, q < LR_VC / 2
+        float2 y1[LR_VC / 2], y2[LR_VC / 2];
+#pragma unroll
+        for (int q = 0; q < LR_VC / 2; ++q) {
+          const int s = g + 2 * q;
+          y1[q] = y2[q] = z2;
+          if (in && s < vc) {
+            if (!a.cplx) {
+              const float *row = a.y + (c0 + s) * a.ld;
+              y1[q].x = __ldg(row + n);
+              y2[q].x = __ldg(row + m);
+            } else {
+              const float2 *row = reinterpret_cast<const float2 *>(a.y) + ((c0 + s) >> 1) * a.ld;
+              y1[q] = __ldg(row + n);
+              y2[q] = __ldg(row + m);
+            }
           }
         }
-        float2 *w = reinterpret_cast<float2 *>(V + i * LR_VS) + s;
-        w[0] = cadd(an, am);
-        w[LR_TN * LR_VS / 2] = csub(an, am);
-        w[LR_TN * LR_VS] = cadd(bn, bm);
-        w[3 * LR_TN * LR_VS / 2] = csub(bn, bm);
+        const float2 pa = in ? a.phA[n] : z2, pam = in ? a.phA[m] : z2, pb = in ? a.phB[n] : z2, pbm = in ? a.phB[m] : z2;
+        const float u = ((float)n - cen) * invN, u2 = u * u;
+        {
+          float p = g ? u : 1.f;
+          const int np = g ? S.npo : S.npe, D = (a.DA > a.DB ? a.DA : a.DB) - g;
+          float *dst = cols + i * S.cs + (g ? 2 * S.nz + S.npe : S.nz);
+          for (int k0 = 0; k0 < np; k0 += 4) {
+            float v[4];
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+              v[kk] = 2 * (k0 + kk) < D ? p : 0.f;
+              p *= u2;
+            }
+            *reinterpret_cast<float4 *>(dst + k0) = make_float4(v[0], v[1], v[2], v[3]);
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < LR_VC / 2; ++q) {
+          const int s = g + 2 * q;
+          if (s < 4 * S.nvt) {
+            float2 an, am, bn, bm;
+            if (!a.cplx) {
+              an = cscale(pa, y1[q].x);
+              am = cscale(pam, y2[q].x);
+              bn = cscale(pb, y1[q].x);
+              bm = cscale(pbm, y2[q].x);
+            } else {
+              const bool cj = ((c0 + s) & 1) != 0;
+              an = cmul(cj ? cconj(pa) : pa, y1[q]);
+              am = cmul(cj ? cconj(pam) : pam, y2[q]);
+              bn = cmul(cj ? cconj(pb) : pb, y1[q]);
+              bm = cmul(cj ? cconj(pbm) : pbm, y2[q]);
+            }
+            float2 *w = reinterpret_cast<float2 *>(V + i * LR_VS) + s;
+            w[0] = cadd(an, am);
+            w[LR_TN * LR_VS / 2] = csub(an, am);
+            w[LR_TN * LR_VS] = cadd(bn, bm);
+            w[3 * LR_TN * LR_VS / 2] = csub(bn, bm);
+          }
+        }
       }
-    }
-    __syncthreads();
-    if (on) {
+      lr_bar_arrive(1 + buf);
+    } else {
+      lr_bar_sync(1 + buf);
+      if (on) {
+        const float *cb = cp + buf * tile_f, *vb = vp + buf * tile_f;
 #pragma unroll 2
-      for (int i = kgi; i < LR_TN; i += S.kg) {
-        const float4 x0 = *reinterpret_cast<const float4 *>(cp + i * S.cs), x1 = *reinterpret_cast<const float4 *>(cp + i * S.cs + 4);
-        const float4 w0 = *reinterpret_cast<const float4 *>(vp + i * LR_VS), w1 = *reinterpret_cast<const float4 *>(vp + i * LR_VS + 4);
-        const float c[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
-        const float2 w[4] = {make_float2(w0.x, w0.y), make_float2(w0.z, w0.w), make_float2(w1.x, w1.y), make_float2(w1.z, w1.w)};
+        for (int i = kgi; i < LR_TN; i += S.kg) {
+          const float4 x0 = *reinterpret_cast<const float4 *>(cb + i * S.cs), x1 = *reinterpret_cast<const float4 *>(cb + i * S.cs + 4);
+          const float4 w0 = *reinterpret_cast<const float4 *>(vb + i * LR_VS), w1 = *reinterpret_cast<const float4 *>(vb + i * LR_VS + 4);
+          const float c[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+          const float2 w[4] = {make_float2(w0.x, w0.y), make_float2(w0.z, w0.w), make_float2(w1.x, w1.y), make_float2(w1.z, w1.w)};
 #pragma unroll
-        for (int r = 0; r < 8; ++r)
+          for (int r = 0; r < 8; ++r)
 #pragma unroll
-          for (int q = 0; q < 4; ++q) fma2(acc[r][q], c[r], w[q]);
+            for (int q = 0; q < 4; ++q) fma2(acc[r][q], c[r], w[q]);
+        }
       }
-    }
-    if (++since == LR_FLUSH) {
-      flush();
-      since = 0;
+      if (t + 2 < t1) lr_bar_arrive(3 + buf);
+      if (++since == LR_FLUSH) {
+        flush();
+        since = 0;
+      }
     }
   }
-  if (since) flush();
+  if (!gen && since) flush();
   __syncthreads();
   // sums of the sample groups in order: red[kg][tile][8 columns][8 floats]
   float *red = lsm;
@@ -205,7 +241,7 @@ __global__ void __launch_bounds__(256, 2) k_coef_gemm(const CoefArgs<float> a, i
     for (int e = 0; e < 64; ++e) red[(kgi * S.ntile + id) * 64 + e] = 0.f;
   }
   __syncthreads();
-  for (int e = tid; e < S.ntile * 64; e += 256) {
+  for (int e = tid; e < S.ntile * 64; e += 512) {
     float s = red[e];
     for (int q = 1; q < S.kg; ++q) s += red[q * S.ntile * 64 + e];
     red[e] = s;
@@ -217,7 +253,7 @@ __global__ void __launch_bounds__(256, 2) k_coef_gemm(const CoefArgs<float> a, i
   };
   const int nq = a.rH + a.DA + a.DB;
   const int vbase[4] = {0, 2 * a.rH + a.DA, 4 * a.rH + 2 * a.DA, 4 * a.rH + 2 * a.DA + a.DB};
-  for (int e = tid; e < vc * nq; e += 256) {
+  for (int e = tid; e < vc * nq; e += 512) {
     const int s = e / nq, k = e % nq;
     const int64_t sig = a.cplx ? (c0 + s) >> 1 : c0 + s;
     const int var = a.cplx ? (int)((c0 + s) & 1) : 0;
