@@ -1026,7 +1026,10 @@ struct DevRunner : Runner {
     const int64_t groups = (rows + sy_rows(rows) - 1) / sy_rows(rows), tiles = ((a.N + 1) / 2 + SY_TN - 1) / SY_TN;
     if (groups > 65535 || a.N < 4 * SY_TN) return 0;
     const int64_t most = std::max<int64_t>((a.N + CORR_BLOCK - 1) / CORR_BLOCK, tc_slices(a.N));
-    return (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(tiles, most), 3 * (int64_t)sms / groups));
+    // ... and more where a thread would otherwise add more than 128 products in a row
+    const int ntile = sy_tiles(a.ncord, a.r - a.ncord) * (sy_rows(rows) / 8), kg = ntile < 16 ? 16 : 256 / ntile;
+    const int64_t want = std::max<int64_t>(3 * (int64_t)sms / groups, (tiles * ((SY_TN / 4 + kg - 1) / kg) * 4 + 127) / 128);
+    return (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(tiles, most), want));
   }
   fst_status sym_c(const ConvArgs<float> &a) override {
     TRY(set_attrs());
