@@ -78,9 +78,9 @@ typedef enum {
  *   eps     tolerance, 0 < eps < 1/2 (Theorem 1, Corollary 2).
  *   stream  stream for the plan-time kernels; the call synchronises it.
  * K need not satisfy the band condition of Corollary 2; T then grows.
- * Cost: the Sturm counts and the tridiagonal LU are serial over the N/2 entries of
- * a reduced matrix, in FP64 (both parities of the window in one batch of targets);
- * on a GB300 about 0.16 s at N = 65536, 2.6 s at N = 2^20 and 10-13 s at N = 2^22.
+ * Cost: the Sturm counts and the eigenvector recurrence are serial over the N/2 entries
+ * of a reduced matrix, in FP64 (both parities of the window in one batch of targets);
+ * on a GB300 about 0.04 s at N = 65536, 0.7 s at N = 2^20 and 2.5 s at N = 2^22.
  * Errors: FST_EINVAL, FST_ENOMEM, FST_ECUDA, FST_ENOCONVERGE.
  */
 fst_status fst_plan(fst_plan_t *out, int64_t N, double W, int64_t K, double eps,
@@ -121,12 +121,12 @@ fst_status fst_plan_export(fst_plan_t plan, int64_t *idx, double *lam, double *D
  *           FST_F64 / FST_C128: the same kernels in FP64.
  * Real signals are processed two at a time as the real and imaginary parts of
  * one complex FFT (B and S_T are real, so they do not mix).
- * FP32: when y is 16-byte aligned, its row stride is a multiple of 16 bytes and the
- * batch has more than 32 signal rows (real signals, or two per complex signal),
- * S_T^T y for the whole batch runs on the tensor cores (TF32 with a hi/lo split,
- * three products); smaller batches use FP32 CUDA-core sums, other layouts mma.sync
- * kernels -- other summation orders, same accuracy.  Results are bit-for-bit
- * repeatable for the same call.
+ * FP32: N <= 8192 takes one CTA per pair.  Longer signals: up to N = 65536, when y is
+ * 16-byte aligned, its row stride is a multiple of 16 bytes and the batch has more than
+ * 32 signal rows (real signals, or two per complex signal), S_T^T y for the whole batch
+ * runs on the tensor cores (TF32 with a hi/lo split, three products); other batches use
+ * FP32 CUDA-core sums over the folded half of S_T -- other summation orders, same
+ * accuracy.  Results are bit-for-bit repeatable for the same call.
  * Errors: FST_EINVAL (NULL pointer, batch < 0, ld < N), FST_ENOMEM, FST_ECUDA,
  * FST_ETIMEOUT (see below).
  * Device waits: every wait of the tensor-core kernel on its own copies and products
@@ -221,8 +221,8 @@ fst_status fst_adi_shifts(int64_t N, int r, double *out);
 /*
  * fst_plan_many -- count plans at once (ragged batches: one plan per signal).
  * Same precomputation as fst_plan for each (N[i], W[i], K[i] or round(2NW) when
- * K is NULL or K[i] < 0, eps[i]), projection operator; the bisection and inverse
- * iteration of all plans' eigen-windows run as one batch of independent targets
+ * K is NULL or K[i] < 0, eps[i]), projection operator; the bisection and the
+ * eigenvectors of all plans' eigen-windows run as one batch of independent targets
  * (about 35 s for 4096 plans with N log-uniform in [1000, 262144] on a GB300).
  * out[count] receives the plans (destroy each with fst_destroy).  On error every
  * plan of the call is freed and out[] is NULL.  Synchronous.
@@ -331,7 +331,7 @@ unsigned long long fst_noalloc_scratch_bytes(void);
  * fst_launch_count   -- number of kernels this process has launched through the
  *                       library so far (plan-time and apply kernels).
  * fst_profile_enable -- on != 0: from now on, every apply-kernel launch and the
- *                       plan-time eigen kernels (bisection, inverse iteration,
+ *                       plan-time eigen kernels (bisection, eigenvectors,
  *                       expansion) are bracketed by CUDA events on their stream;
  *                       clears earlier records.  on == 0 stops recording (and clears).
  * fst_profile_count  -- number of recorded launches.

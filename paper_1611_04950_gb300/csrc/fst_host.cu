@@ -421,7 +421,10 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
       TRY(ensure_ws(p, ws_need(Lp, false, (int)p->rpad, false)));
       return run_conv<T>(R, Lp, a, npairs, p->ws);
     }
-    const F64Plan f64 = dbl ? f64_plan(p, npairs, cplx, batch, full) : F64Plan();
+    F64Plan f64 = dbl ? f64_plan(p, npairs, cplx, batch, full) : F64Plan();
+    // inside a caller's stream capture nothing can be allocated: without enough workspace the generic
+    // kernels run, which need less of it (none for the single-CTA lengths)
+    if (f64.on && f64.inter_b + f64.part_b + f64.acoef_b > p->ws_bytes && R->user_stream_capturing()) f64.on = false;
     const size_t slot = f64.on ? f64.inter_b : ws_need(Lc, dbl, (int)p->rpad, false);
     const size_t extra = f64.on ? f64.part_b + f64.acoef_b : sep_b;
     auto run = [&]() { return f64.on ? run_f64(p, f64, a, npairs, (char *)p->ws) : run_conv<T>(R, Lc, a, npairs, p->ws); };

@@ -18,6 +18,7 @@ from oracle import fst_oracle as O  # noqa: E402
     (511, 0.2, 1e-6, None, 3, False), (257, 0.1, 1e-3, None, 1, True), (1000, 1 / 64, 1e-8, None, 5, False),
     (2047, 0.25, 1e-8, None, 9, True), (4096, 1 / 16, 1e-6, None, 2, False), (4097, 0.2, 1e-6, None, 33, False),
     (8191, 0.05, 1e-4, None, 2, True), (9001, 0.1, 1e-6, None, 7, False), (20011, 0.25, 1e-8, None, 3, True),
+    (8000, 0.1, 1e-6, None, 90, False), (16001, 0.1, 1e-6, None, 40, True),
     (65536, 1 / 8, 1e-4, None, 5, False), (100003, 0.03, 1e-6, None, 2, True), (600, 0.2, 1e-6, 40, 17, False)])
 def test_fp64_against_oracle(N, W, eps, K, batch, cplx):
     if not torch.cuda.is_available():
@@ -39,3 +40,20 @@ def test_fp64_against_oracle(N, W, eps, K, batch, cplx):
     b = p.apply_prolate(yd).cpu().numpy()
     z = (o.S_T @ (o.D[:, None] * (o.S_T.T @ y.numpy().T))).T
     assert np.all(np.linalg.norm(b + z - ref, axis=1) < 1e-12 * nrm)
+
+
+def test_fp64_in_a_stream_capture_without_workspace():
+    # nothing can be allocated while a caller records a graph: a plan that has not run yet takes the
+    # kernels that need no workspace
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    p, q = F.Plan(3000, 0.2, eps=1e-6), F.Plan(3000, 0.2, eps=1e-6)
+    y = workloads.gaussian(3, 3000, seed=1).to("cuda")
+    out = torch.empty_like(y)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        p.project(y, out=out)
+    g.replay()
+    torch.cuda.synchronize()
+    ref = q.project(y)
+    assert float((out - ref).norm()) < 1e-12 * float(y.norm())
