@@ -223,7 +223,7 @@ fst_status fst_adi_shifts(int64_t N, int r, double *out);
  * Same precomputation as fst_plan for each (N[i], W[i], K[i] or round(2NW) when
  * K is NULL or K[i] < 0, eps[i]), projection operator; the bisection and the
  * eigenvectors of all plans' eigen-windows run as one batch of independent targets
- * (about 35 s for 4096 plans with N log-uniform in [1000, 262144] on a GB300).
+ * (about 21 s for 4096 plans with N log-uniform in [1000, 262144] on a GB300).
  * out[count] receives the plans (destroy each with fst_destroy).  On error every
  * plan of the call is freed and out[] is NULL.  Synchronous.
  */
