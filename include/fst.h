@@ -127,6 +127,12 @@ fst_status fst_plan_export(fst_plan_t plan, int64_t *idx, double *lam, double *D
  * runs on the tensor cores (TF32 with a hi/lo split, three products); other batches use
  * FP32 CUDA-core sums over the folded half of S_T -- other summation orders, same
  * accuracy.  Results are bit-for-bit repeatable for the same call.
+ * Stream capture: on a capturing stream the call allocates nothing and records its
+ * kernels.  N <= 8192 in FP32 and N <= 4096 in FP64 use no workspace there (FP64: one CTA
+ * per pair, a kernel that is slower than that of a direct call).  Longer signals use the
+ * plan's workspace as an earlier call of at least that size left it, and a recorded graph
+ * is valid only until a larger call on the plan (fst_project, fst_apply_prolate,
+ * fst_coeffs, fst_expand) replaces it: record after the largest call.
  * Errors: FST_EINVAL (NULL pointer, batch < 0, ld < N), FST_ENOMEM, FST_ECUDA,
  * FST_ETIMEOUT (see below).
  * Device waits: every wait of the tensor-core kernel on its own copies and products

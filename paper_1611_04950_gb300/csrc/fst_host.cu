@@ -422,9 +422,12 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
       return run_conv<T>(R, Lp, a, npairs, p->ws);
     }
     F64Plan f64 = dbl ? f64_plan(p, npairs, cplx, batch, full) : F64Plan();
-    // inside a caller's stream capture nothing can be allocated: without enough workspace the generic
-    // kernels run, which need less of it (none for the single-CTA lengths)
-    if (f64.on && f64.inter_b + f64.part_b + f64.acoef_b > p->ws_bytes && R->user_stream_capturing()) f64.on = false;
+    // inside a caller's stream capture nothing can be allocated, and what is recorded keeps pointing at
+    // the workspace, which a later larger call frees: the single-CTA lengths take the generic kernel,
+    // which needs none (whatever the plan has run before, so the same call records the same kernels).
+    // Longer ones need a workspace with any kernels; theirs are the generic ones where it is too small.
+    if (f64.on && R->user_stream_capturing() &&
+        (p->lay64.small || f64.inter_b + f64.part_b + f64.acoef_b > p->ws_bytes)) f64.on = false;
     const size_t slot = f64.on ? f64.inter_b : ws_need(Lc, dbl, (int)p->rpad, false);
     const size_t extra = f64.on ? f64.part_b + f64.acoef_b : sep_b;
     auto run = [&]() { return f64.on ? run_f64(p, f64, a, npairs, (char *)p->ws) : run_conv<T>(R, Lc, a, npairs, p->ws); };

@@ -57,3 +57,40 @@ def test_fp64_in_a_stream_capture_without_workspace():
     torch.cuda.synchronize()
     ref = q.project(y)
     assert float((out - ref).norm()) < 1e-12 * float(y.norm())
+
+
+def _captured(p, y):
+    out = torch.empty_like(y)
+    p.project(torch.zeros_like(y[:1]))          # first-call set-up happens before the recording
+    torch.cuda.synchronize()
+    n0 = F.fst_launch_count()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        p.project(y, out=out)
+    return g, out, F.fst_launch_count() - n0
+
+
+@pytest.mark.parametrize("batch,cplx", [(3, False), (2, True), (40, False)])
+def test_fp64_short_signals_captured_without_the_workspace(batch, cplx):
+    # single-CTA lengths: a caller's graph must not point at the plan's workspace, which a later
+    # larger call frees, and must not depend on what the plan has run before
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    p, q = F.Plan(3000, 0.2, eps=1e-6), F.Plan(3000, 0.2, eps=1e-6)
+    y = workloads.gaussian(batch, 3000, seed=1, complex_=cplx).to("cuda")
+    p.project(y)
+    g, out, launches = _captured(p, y)
+    assert launches == 1                        # the whole projection in one launch, no scratch
+    big = workloads.gaussian(400, 3000, seed=2).to("cuda")
+    p.project(big)                              # moves the workspace
+    out.zero_()
+    g.replay()
+    torch.cuda.synchronize()
+    first = out.clone()
+    cold = torch.empty_like(y)
+    gq = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(gq):
+        q.project(y, out=cold)
+    gq.replay()
+    torch.cuda.synchronize()
+    assert torch.equal(first, cold)
