@@ -308,7 +308,8 @@ struct F64Plan {
   int64_t group = 0;                                 // pairs per launch group
   size_t inter_b = 0, part_b = 0, acoef_b = 0;
 };
-static F64Plan f64_plan(fst_plan_t p, int64_t npairs, bool cplx, int64_t batch, bool full) {
+// room > 0: bytes that are there; the launch groups shrink to fit (they do not change the arithmetic)
+static F64Plan f64_plan(fst_plan_t p, int64_t npairs, bool cplx, int64_t batch, bool full, size_t room) {
   F64Plan f;
   // (rows beyond 4 * 65535 do not fit the grid of the S_T a pass: the generic kernels take those)
   if (!p->R->device() || p->log2M < 10 || p->log2M > 18 || !p->cpar || (cplx ? 2 : 1) * batch > 4 * 65535) return f;
@@ -326,6 +327,12 @@ static F64Plan f64_plan(fst_plan_t p, int64_t npairs, bool cplx, int64_t batch, 
     f.nchunk = (int)((H + f.chunk - 1) / f.chunk);
     f.part_b = (size_t)f.nchunk * rows * p->rpad * sizeof(double);
     f.acoef_b = (size_t)rows * p->rpad * sizeof(double);
+  }
+  if (room > 0 && f.inter_b + f.part_b + f.acoef_b > room) {
+    const size_t pair_b = (size_t)16 << p->log2M, rest = f.part_b + f.acoef_b;
+    f.group = rest < room ? (int64_t)((room - rest) / pair_b) : 0;
+    f.inter_b = (size_t)f.group * pair_b;
+    f.on = f.group > 0;
   }
   return f;
 }
@@ -421,13 +428,15 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
       TRY(ensure_ws(p, ws_need(Lp, false, (int)p->rpad, false)));
       return run_conv<T>(R, Lp, a, npairs, p->ws);
     }
-    F64Plan f64 = dbl ? f64_plan(p, npairs, cplx, batch, full) : F64Plan();
     // inside a caller's stream capture nothing can be allocated, and what is recorded keeps pointing at
     // the workspace, which a later larger call frees: the single-CTA lengths take the generic kernel,
-    // which needs none (whatever the plan has run before, so the same call records the same kernels).
-    // Longer ones need a workspace with any kernels; theirs are the generic ones where it is too small.
-    if (f64.on && R->user_stream_capturing() &&
-        (p->lay64.small || f64.inter_b + f64.part_b + f64.acoef_b > p->ws_bytes)) f64.on = false;
+    // which needs none.  Longer ones need a workspace with any kernels and make do with what is there,
+    // so that the same call records the same arithmetic whatever the plan has run before (a batch whose
+    // coefficients alone fill it: the generic kernels).
+    const bool recording = dbl && R->user_stream_capturing();
+    F64Plan f64;
+    if (dbl && !(recording && p->lay64.small))
+      f64 = f64_plan(p, npairs, cplx, batch, full, recording ? std::max<size_t>(1, p->ws_bytes) : 0);
     const size_t slot = f64.on ? f64.inter_b : ws_need(Lc, dbl, (int)p->rpad, false);
     const size_t extra = f64.on ? f64.part_b + f64.acoef_b : sep_b;
     auto run = [&]() { return f64.on ? run_f64(p, f64, a, npairs, (char *)p->ws) : run_conv<T>(R, Lc, a, npairs, p->ws); };

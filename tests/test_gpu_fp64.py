@@ -94,3 +94,24 @@ def test_fp64_short_signals_captured_without_the_workspace(batch, cplx):
     gq.replay()
     torch.cuda.synchronize()
     assert torch.equal(first, cold)
+
+
+def test_fp64_captured_whatever_ran_before():
+    # longer lengths: a workspace left by a smaller call holds fewer pairs at a time, not other sums
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    y = workloads.gaussian(32, 8000, seed=5).to("cuda")
+    outs = []
+    for warm in (32, 16):
+        p = F.Plan(8000, 0.2, eps=1e-6)
+        p.project(y[:warm].clone())
+        out = torch.empty_like(y)
+        torch.cuda.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            p.project(y, out=out)
+        g.replay()
+        torch.cuda.synchronize()
+        outs.append((out, p))
+    assert torch.equal(outs[0][0], outs[1][0])
+    assert torch.equal(outs[0][0], outs[0][1].project(y))
