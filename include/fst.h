@@ -126,7 +126,8 @@ fst_status fst_plan_export(fst_plan_t plan, int64_t *idx, double *lam, double *D
  * 32 signal rows (real signals, or two per complex signal), S_T^T y for the whole batch
  * runs on the tensor cores (TF32 with a hi/lo split, three products); other batches use
  * FP32 CUDA-core sums over the folded half of S_T -- other summation orders, same
- * accuracy.  Results are bit-for-bit repeatable for the same call.
+ * accuracy.  The number of partial sums follows the batch in FP64 (N > 256) and in the
+ * folded form.  Results are bit-for-bit repeatable for the same call.
  * Stream capture: on a capturing stream the call allocates nothing and records its
  * kernels.  N <= 8192 in FP32 and N <= 4096 in FP64 use no workspace there (FP64: one CTA
  * per pair, a kernel that is slower than that of a direct call).  Longer signals use the
@@ -154,7 +155,8 @@ fst_status fst_project(fst_plan_t plan, const void *y, void *out, int64_t batch,
  * chunks on `stream`, overlapping copies with compute (four chunks in flight; the
  * first and last chunks are a quarter of the others); returns after the result is
  * in `out` (synchronous).  Pinned host memory gives the full link bandwidth.  The
- * results are bit-for-bit those of fst_project on the whole batch.  Device scratch:
+ * results are bit-for-bit those of fst_project on the whole batch, contiguous and 16-byte
+ * aligned in device memory (every choice goes by the whole batch, not the chunk).  Device scratch:
  * eight chunk buffers of up to FST_HOST_CHUNK_MB (default 64) MiB, allocated on the first
  * call of a thread and kept for its later calls.
  */

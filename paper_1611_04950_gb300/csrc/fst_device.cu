@@ -1022,7 +1022,7 @@ struct DevRunner : Runner {
   // chunks of S_T^T y: about three blocks per SM in all (two are resident), at least a tile each, and
   // no more partials than the scratch of the other forms holds (CORR_BLOCK samples each)
   int sym_chunks(const ConvArgs<float> &a) override {
-    const int64_t rows = a.cplx ? 2 * a.batch : a.batch;
+    const int64_t rows = a.rows_all;
     const int64_t groups = (rows + sy_rows(rows) - 1) / sy_rows(rows), tiles = ((a.N + 1) / 2 + SY_TN - 1) / SY_TN;
     if (groups > 65535 || a.N < 4 * SY_TN) return 0;
     const int64_t most = std::max<int64_t>((a.N + CORR_BLOCK - 1) / CORR_BLOCK, tc_slices(a.N));
@@ -1034,7 +1034,7 @@ struct DevRunner : Runner {
   fst_status sym_c(const ConvArgs<float> &a) override {
     TRY(set_attrs());
     const int64_t rows = a.cplx ? 2 * a.batch : a.batch;
-    const int RB = sy_rows(rows);
+    const int RB = sy_rows(a.rows_all);
     dim3 grid((unsigned)a.nkb, (unsigned)((rows + RB - 1) / RB));
     const size_t smem = sy_smem(a.ncord, a.r - a.ncord, RB);
     auto go = [&](auto kernel) { PROF("k_sym_c", a.npairs, (kernel<<<grid, 256, smem, cur>>>(a, a.cord, a.ncord, a.nkb))); };
@@ -1515,7 +1515,7 @@ extern "C" fst_status fst_project_host(fst_plan_t p, const void *y, void *out, i
     CU(cudaMemcpyAsync(hp.din[k], (const char *)y + b0 * sig_bytes, bytes, cudaMemcpyHostToDevice, hp.cin), "h2d");
     CU(cudaEventRecord(hp.in_done[k], hp.cin), "event");
     CU(cudaStreamWaitEvent(sc, hp.in_done[k], 0), "wait");
-    fst_status s = run_apply(p, hp.din[k], hp.dout[k], nb, 0, dtype, true);
+    fst_status s = run_apply(p, hp.din[k], hp.dout[k], nb, 0, dtype, true, batch);
     if (s != FST_OK) return s;
     CU(cudaEventRecord(hp.comp_done[k], sc), "event");
     CU(cudaStreamWaitEvent(hp.cout, hp.comp_done[k], 0), "wait");

@@ -157,8 +157,10 @@ __device__ __forceinline__ int64_t f64_elem(const ConvArgs<double> &a, int64_t r
 }
 
 // c partials: block (chunk of ch folded samples, RG rows), 256 threads.  Thread (slice, row, j) sums
-// s_j(n) (y(n) +- y(N-1-n)) over the samples of its slice; the slices are added in order.  The
-// folded rows and S_T rows pass through shared memory 32 samples at a time.  64 columns a round.
+// s_j(n) (y(n) +- y(N-1-n)) over the samples of its slice; the slices are added in order.  The folded
+// rows and S_T rows pass through shared memory 32 samples at a time.  64 columns a round, and of the
+// rows as many as 256 threads take; the number of slices goes by the rows of the whole call, so every
+// row adds in the same order wherever it lies in its block.
 // part: [chunk][row][rpad]
 constexpr int F64_RG = 8, F64_SUB = 32, F64_JB = 64;
 __global__ void __launch_bounds__(256) k_f64_corr(const ConvArgs<double> a, const unsigned char *cpar, int ch,
@@ -170,13 +172,13 @@ __global__ void __launch_bounds__(256) k_f64_corr(const ConvArgs<double> a, cons
   const int nr = (int)(rows - row0 < F64_RG ? rows - row0 : F64_RG);
   for (int j0 = 0; j0 < a.r; j0 += F64_JB) {
     const int nj = a.r - j0 < F64_JB ? a.r - j0 : F64_JB;
-    const int outs = nr * nj;                       // up to 512: two rounds of row halves
-    for (int o0 = 0; o0 < outs; o0 += 256) {
-      const int no = outs - o0 < 256 ? outs - o0 : 256;
-      const int nsl = 256 / no;
-      const int o = o0 + threadIdx.x % no, sl = threadIdx.x / no;
-      const int rr = o / nj, j = o % nj;
-      const bool on = sl < nsl, odd = on && cpar[j0 + j];
+    const int rg = (int)(a.rows_all < F64_RG ? a.rows_all : F64_RG);
+    const int rpr = rg * nj <= 256 ? rg : (rg + 1) / 2;   // rows a round
+    const int no = rpr * nj, nsl = 256 / no;
+    for (int q0 = 0; q0 < nr; q0 += rpr) {
+      const int o = threadIdx.x % no, sl = threadIdx.x / no;
+      const int rr = q0 + o / nj, j = o % nj;
+      const bool on = sl < nsl && rr < nr, odd = on && cpar[j0 + j];
       double acc = 0.0;
       for (int64_t m0 = n0; m0 < n1; m0 += F64_SUB) {
         const int ns = (int)(n1 - m0 < F64_SUB ? n1 - m0 : F64_SUB);
@@ -197,7 +199,7 @@ __global__ void __launch_bounds__(256) k_f64_corr(const ConvArgs<double> a, cons
       __syncthreads();
       red[threadIdx.x] = acc;
       __syncthreads();
-      if (threadIdx.x < no) {
+      if (threadIdx.x < no && rr < nr) {
         double s = acc;
         for (int q = 1; q < nsl; ++q) s += red[q * no + threadIdx.x];
         part[((int64_t)blockIdx.x * rows + row0 + rr) * a.rpad + j0 + j] = s;

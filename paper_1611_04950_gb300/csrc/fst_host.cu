@@ -162,7 +162,7 @@ static bool tc_usable(const ConvArgs<float> &a) {
 
 // S_T^T y for every pair into sc.part, then a = scale o (sum of the partials) into sc.acoef
 static fst_status corr_coefficients(Runner *R, ConvArgs<float> &sc, const float *scale) {
-  const int64_t rows = sc.cplx ? 2 * sc.batch : sc.batch;
+  const int64_t rows = sc.rows_all;
   const int combos = (int)((rows + 3) / 4) * (sc.rpad / 8);
   // folded form on CUDA cores (half of S_T and of the FMAs) where the plan has the K-major S_T^T,
   // except batches of more than 32 rows that the tcgen05 kernel can address at P <= 32: there it is
@@ -210,7 +210,7 @@ static fst_status run_conv(Runner *R, const Layout &L, ConvArgs<T> a, int64_t np
   const ConvArgs<float> &af = *reinterpret_cast<const ConvArgs<float> *>(&a);
   // (at P = 8 and 17 to 64 rows no tensor map can address, the column pass's own products are the
   // faster ones: 33 rows of 9001 samples 21.1 us, folded 23.6)
-  const int64_t nrows = a.cplx ? 2 * a.batch : a.batch;
+  const int64_t nrows = a.rows_all;
   const bool sym = af.STt && af.cord && !plain_mode() && !(L.fast && L.log2P == 3 && nrows > 16 && nrows <= 64);
   const bool split = want && (L.split_corr || tc || sym);
   ConvArgs<float> sc{};
@@ -301,7 +301,8 @@ static void odd_bits(fst_plan_t p, unsigned *odd) {
 
 // FP64 four-step path of fst_fast64.cuh: M = 2^10 .. 2^18.  The split is P = 32, or for batches whose
 // rows fill the GPU that of the plan's FP64 layout (rows of at least 2048 points, the faster row
-// kernel).  The plan's spectrum keeps its own order (natural up to M = 2^13).
+// kernel).  The plan's spectrum keeps its own order (natural up to M = 2^13).  Split and partials go by
+// the rows of the whole call (rows_all), so that a host-buffer chunk gets the bits of the whole batch.
 struct F64Plan {
   bool on = false;
   int log2P = 0, log2Q = 0, chunk = 0, nchunk = 0;   // chunk: folded samples per partial of S_T^T y
@@ -309,19 +310,20 @@ struct F64Plan {
   size_t inter_b = 0, part_b = 0, acoef_b = 0;
 };
 // room > 0: bytes that are there; the launch groups shrink to fit (they do not change the arithmetic)
-static F64Plan f64_plan(fst_plan_t p, int64_t npairs, bool cplx, int64_t batch, bool full, size_t room) {
+static F64Plan f64_plan(fst_plan_t p, const ConvArgs<double> &a, int64_t npairs, bool full, size_t room) {
   F64Plan f;
+  const int64_t all = a.rows_all;
   // (rows beyond 4 * 65535 do not fit the grid of the S_T a pass: the generic kernels take those)
-  if (!p->R->device() || p->log2M < 10 || p->log2M > 18 || !p->cpar || (cplx ? 2 : 1) * batch > 4 * 65535) return f;
+  if (!p->R->device() || p->log2M < 10 || p->log2M > 18 || !p->cpar || all > 4 * 65535) return f;
   f.on = true;
   f.log2P = 5;
-  if (!p->lay64.small && (npairs << p->lay64.log2P) >= 2 * p->R->sm_count()) f.log2P = p->lay64.log2P;
+  if (!p->lay64.small && (((all + 1) / 2) << p->lay64.log2P) >= 2 * p->R->sm_count()) f.log2P = p->lay64.log2P;
   f.log2Q = p->log2M - f.log2P;
   f.group = std::max<int64_t>(1, std::min<int64_t>(npairs, chunk_bytes_target() >> (p->log2M + 4)));
   f.inter_b = ((size_t)f.group << (p->log2M + 4));
   if (full && p->r > 0) {
     // partials over chunks of at least one 32-sample tile; about four blocks per SM in all
-    const int64_t rows = cplx ? 2 * batch : batch, H = (p->N + 1) / 2, rg = (rows + 7) / 8;
+    const int64_t rows = a.cplx ? 2 * a.batch : a.batch, H = (p->N + 1) / 2, rg = (all + 7) / 8;
     const int64_t want = std::max<int64_t>(1, 4 * (int64_t)p->R->sm_count() / rg);
     f.chunk = (int)(((H + want - 1) / want + 31) / 32 * 32);
     f.nchunk = (int)((H + f.chunk - 1) / f.chunk);
@@ -381,7 +383,7 @@ static fst_status run_f64(fst_plan_t, const F64Plan &, ConvArgs<float>, int64_t,
 template <typename T>
 static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64_t ld, bool cplx, bool full,
                           const T *spec, const T *ST, const T *D, const Layout &L0, void *ext_ws,
-                          size_t ext_bytes) {
+                          size_t ext_bytes, int64_t whole) {
   ConvArgs<T> a{};
   a.y = y;
   a.out = out;
@@ -412,6 +414,7 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
   a.D = D;
   a.tw = plan_tw<T>(p);
   a.mode = full ? MODE_FULL : MODE_CONV;
+  a.rows_all = (cplx ? 2 : 1) * std::max(batch, whole);
   const int64_t npairs = cplx ? batch : (batch + 1) / 2;
   const bool dbl = sizeof(T) == 8;
   const bool sep = (L0.split_corr || (p->STt && !L0.small && !dbl)) && full && p->r > 0;
@@ -436,7 +439,7 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
     const bool recording = dbl && R->user_stream_capturing();
     F64Plan f64;
     if (dbl && !(recording && p->lay64.small))
-      f64 = f64_plan(p, npairs, cplx, batch, full, recording ? std::max<size_t>(1, p->ws_bytes) : 0);
+      f64 = f64_plan(p, *reinterpret_cast<const ConvArgs<double> *>(&a), npairs, full, recording ? std::max<size_t>(1, p->ws_bytes) : 0);
     const size_t slot = f64.on ? f64.inter_b : ws_need(Lc, dbl, (int)p->rpad, false);
     const size_t extra = f64.on ? f64.part_b + f64.acoef_b : sep_b;
     auto run = [&]() { return f64.on ? run_f64(p, f64, a, npairs, (char *)p->ws) : run_conv<T>(R, Lc, a, npairs, p->ws); };
@@ -448,7 +451,7 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
     }
     // whole apply as one cached CUDA graph (two overlapping lanes of launch groups)
     for (auto &e : p->graphs)
-      if (e.y == (const void *)y && e.out == (void *)out && e.batch == batch && e.ld == ld &&
+      if (e.y == (const void *)y && e.out == (void *)out && e.batch == batch && e.ld == ld && e.rows_all == a.rows_all &&
           e.dtype == (int)(cplx ? 1 : 0) + (dbl ? 2 : 0) && e.full == full)
         return R->graph_launch(e.exec, e.nodes);
     TRY(ensure_ws(p, 2 * slot + 256 + extra));
@@ -467,8 +470,8 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
       R->graph_destroy(p->graphs.front().exec);
       p->graphs.erase(p->graphs.begin());
     }
-    p->graphs.push_back({(const void *)y, (void *)out, batch, ld, (int)(cplx ? 1 : 0) + (dbl ? 2 : 0), full, exec,
-                         nodes});
+    p->graphs.push_back({(const void *)y, (void *)out, batch, ld, a.rows_all, (int)(cplx ? 1 : 0) + (dbl ? 2 : 0), full,
+                         exec, nodes});
     return R->graph_launch(exec, nodes);
   }
   // caller-provided scratch: shrink the launch group until it fits
@@ -488,7 +491,7 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
 }
 
 fst_status run_apply_ws(fst_plan_t p, const void *y, void *out, int64_t batch, int64_t ld, int dtype, bool full,
-                        void *ws, size_t ws_bytes) {
+                        void *ws, size_t ws_bytes, int64_t whole) {
   if (!p) return fail(FST_EINVAL, "plan is NULL");
   if (batch < 0) return fail(FST_EINVAL, "batch < 0");
   if (batch == 0) return FST_OK;
@@ -499,23 +502,24 @@ fst_status run_apply_ws(fst_plan_t p, const void *y, void *out, int64_t batch, i
   switch (dtype) {
     case FST_F32:
       return apply_t<float>(p, (const float *)y, (float *)out, batch, ld, false, full, p->spec32, p->ST32, p->D32,
-                            p->lay32, ws, ws_bytes);
+                            p->lay32, ws, ws_bytes, whole);
     case FST_C64:
       return apply_t<float>(p, (const float *)y, (float *)out, batch, ld, true, full, p->spec32, p->ST32, p->D32,
-                            p->lay32, ws, ws_bytes);
+                            p->lay32, ws, ws_bytes, whole);
     case FST_F64:
       return apply_t<double>(p, (const double *)y, (double *)out, batch, ld, false, full, p->spec64, p->ST64,
-                             p->D64, p->lay64, ws, ws_bytes);
+                             p->D64, p->lay64, ws, ws_bytes, whole);
     case FST_C128:
       return apply_t<double>(p, (const double *)y, (double *)out, batch, ld, true, full, p->spec64, p->ST64,
-                             p->D64, p->lay64, ws, ws_bytes);
+                             p->D64, p->lay64, ws, ws_bytes, whole);
     default:
       return fail(FST_EINVAL, "unknown dtype");
   }
 }
 
-fst_status run_apply(fst_plan_t p, const void *y, void *out, int64_t batch, int64_t ld, int dtype, bool full) {
-  return run_apply_ws(p, y, out, batch, ld, dtype, full, nullptr, 0);
+fst_status run_apply(fst_plan_t p, const void *y, void *out, int64_t batch, int64_t ld, int dtype, bool full,
+                     int64_t whole) {
+  return run_apply_ws(p, y, out, batch, ld, dtype, full, nullptr, 0, whole);
 }
 
 // ---------------------------------------------------------------------------
@@ -1497,6 +1501,7 @@ static fst_status coeffs_t(fst_plan_t p, const T *y, c2<T> *out, int64_t batch, 
     ca.ld = ld;
     ca.batch = batch;
     ca.cplx = cplx ? 1 : 0;
+    ca.rows_all = (cplx ? 2 : 1) * batch;
     ca.N = N;
     ca.r = (int)p->r;
     ca.rpad = (int)p->rpad;

@@ -224,7 +224,7 @@ struct fst_plan_s {
   struct GraphEntry {
     const void *y;
     void *out;
-    int64_t batch, ld;
+    int64_t batch, ld, rows_all;
     int dtype;
     bool full;
     void *exec;
@@ -239,12 +239,14 @@ fst_status fail(fst_status st, const std::string &msg);
 // build a plan with the given runner (takes ownership of R)
 fst_status build_plan(Runner *R, fst_plan_t *out, int64_t N, double W, int64_t K, double eps, int op,
                       double alpha);
-// B y (+ correction when full) for `batch` signals in runner memory
-fst_status run_apply(fst_plan_t p, const void *y, void *out, int64_t batch, int64_t ld, int dtype, bool full);
+// B y (+ correction when full) for `batch` signals in runner memory; whole: signals of the call that
+// these are a part of (0: these are all), whose sums they then get bit for bit
+fst_status run_apply(fst_plan_t p, const void *y, void *out, int64_t batch, int64_t ld, int dtype, bool full,
+                     int64_t whole = 0);
 // as run_apply with caller-provided scratch `ws` of ws_bytes (nullptr: the plan's own,
 // allocated on demand); with caller scratch nothing is allocated
 fst_status run_apply_ws(fst_plan_t p, const void *y, void *out, int64_t batch, int64_t ld, int dtype, bool full,
-                        void *ws, size_t ws_bytes);
+                        void *ws, size_t ws_bytes, int64_t whole = 0);
 void destroy_plan(fst_plan_t p);
 bool profiling_enabled();   // per-launch event timing is on (fst_profile_enable)
 // Device buffers and launch choices of one ragged signature (owned by the caller): the first

@@ -141,6 +141,8 @@ template <typename T> struct ConvArgs {
   unsigned odd[4];    // columns as bits (STt then holds its K-major copy, rows tc_Npad apart)
   const c2<T> *exp_c; // forward transform of T1 c: coefficient vectors, exp_kp apart, bins -exp_h..exp_h first
   int64_t exp_kp, exp_h;
+  int64_t rows_all;   // signal rows (real signals, or two per complex one) of the whole call: what every choice
+                      // that changes a summation order goes by; more than the batch has in a host-buffer chunk
   const RPair<T> *rp; // ragged batch: per pair slot signal, length and spectrum (else nullptr)
   int two_spec;       // ragged real slots hold two signals with their own spectra (pass B pairs rows)
 };
