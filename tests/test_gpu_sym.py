@@ -36,3 +36,26 @@ def test_folded_correction(N, W, eps, batch, cplx):
     wide.copy_(yd)
     got = p.project(wide, out=wide)                      # in place
     assert np.all(np.linalg.norm(got.cpu().numpy()[pick] - ref, axis=1) < 1e-5 * nrm[pick])
+
+
+@pytest.mark.parametrize("N,W,eps,batch,cplx", [(40000, 0.25, 1e-8, 64, False), (65536, 0.2, 1e-8, 17, True),
+                                                (8196, 0.2, 1e-9, 33, False)])
+def test_tensor_core_correction_rank_33_to_64(N, W, eps, batch, cplx):
+    # more than 32 addressable rows, N <= 65536, two column tiles of 32: the tcgen05 sums
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    p = F.Plan(N, W, eps=eps)
+    o = O.make_plan(N, W, p.K, eps)
+    assert p.r == o.r and 32 < p.r <= 64
+    y = workloads.gaussian(batch, N, seed=batch, complex_=cplx).to(torch.complex64 if cplx else torch.float32)
+    pick = sorted({0, batch // 2, batch - 1})
+    ref = O.fast_project(o, y.numpy()[pick].astype(np.complex128 if cplx else np.float64).T).T
+    yd = y.to("cuda")
+    F.fst_profile_enable(True)
+    out = p.project(yd)
+    names = {r[0] for r in F.fst_profile_records()}
+    F.fst_profile_enable(False)
+    assert "k_corr_tc" in names
+    nrm = np.linalg.norm(y.numpy(), axis=1)
+    assert np.all(np.linalg.norm(out.cpu().numpy()[pick] - ref, axis=1) < 1e-5 * nrm[pick])
+    assert torch.equal(p.project(yd), out)
