@@ -128,6 +128,9 @@ fst_status fst_plan_export(fst_plan_t plan, int64_t *idx, double *lam, double *D
  * FP32 CUDA-core sums over the folded half of S_T -- other summation orders, same
  * accuracy.  The number of partial sums follows the batch in FP64 (N > 256) and in the
  * folded form.  Results are bit-for-bit repeatable for the same call.
+ * Workspace: kept by the plan and grown on demand, at most two launch groups of 128 MiB
+ * (FST_CHUNK_MB) plus partial sums.  FP32 of N <= 8192 needs none.  FP64 of N <= 4096 does
+ * without one, on slower kernels, where the device has no room for it.
  * Stream capture: on a capturing stream the call allocates nothing and records its
  * kernels.  N <= 8192 in FP32 and N <= 4096 in FP64 use no workspace there (FP64: one CTA
  * per pair, a kernel that is slower than that of a direct call).  Longer signals use the

@@ -38,6 +38,13 @@ int fst_plan_is_emulated(fst_plan_t plan);
  */
 fst_status fst_test_tc_stall(int launches, double limit_s);
 
+/*
+ * Test hook for calls on a full device: the next `allocations` device allocations of the
+ * library (plans, workspaces, ragged batches) fail as cudaMalloc does without memory, and
+ * allocate nothing.  0 ends it.  Errors: FST_EINVAL (allocations < 0).
+ */
+fst_status fst_test_alloc_fail(int allocations);
+
 #ifdef __cplusplus
 }
 #endif

@@ -500,6 +500,15 @@ bool tc_stall_take() {
   return false;
 }
 
+// test hook (fst_test_alloc_fail): the next g_alloc_fail device allocations report a full device
+static std::atomic<int> g_alloc_fail{0};
+static bool alloc_fail_take() {
+  int v = g_alloc_fail.load();
+  while (v > 0)
+    if (g_alloc_fail.compare_exchange_weak(v, v - 1)) return true;
+  return false;
+}
+
 static inline int grid_for(int64_t n, int block) {
   int64_t g = (n + block - 1) / block;
   return (int)std::max<int64_t>(1, std::min<int64_t>(g, 152 * 32));
@@ -671,8 +680,10 @@ struct DevRunner : Runner {
 
   fst_status alloc(void **p, size_t bytes) override {
     *p = nullptr;
-    CU(cudaMalloc(p, std::max<size_t>(bytes, 16)), "cudaMalloc");
-    return FST_OK;
+    const cudaError_t e = alloc_fail_take() ? cudaErrorMemoryAllocation : cudaMalloc(p, std::max<size_t>(bytes, 16));
+    if (e == cudaSuccess) return FST_OK;
+    cudaGetLastError();   // a caller that goes on without this memory must not find the error at its next launch
+    return cuda_fail(e, "cudaMalloc");
   }
   void release(void *p) override {
     if (p) cudaFree(p);
@@ -1688,6 +1699,12 @@ extern "C" fst_status fst_ragged_tuning(const fst_plan_t *plans, const void *con
       return FST_OK;
     }
   return fail(FST_EINVAL, "no ragged call with this signature has run");
+}
+
+extern "C" fst_status fst_test_alloc_fail(int allocations) {
+  if (allocations < 0) return fail(FST_EINVAL, "bad allocation count");
+  fst::g_alloc_fail.store(allocations);
+  return FST_OK;
 }
 
 extern "C" fst_status fst_test_tc_stall(int launches, double limit_s) {

@@ -440,13 +440,22 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
     F64Plan f64;
     if (dbl && !(recording && p->lay64.small))
       f64 = f64_plan(p, *reinterpret_cast<const ConvArgs<double> *>(&a), npairs, full, recording ? std::max<size_t>(1, p->ws_bytes) : 0);
-    const size_t slot = f64.on ? f64.inter_b : ws_need(Lc, dbl, (int)p->rpad, false);
-    const size_t extra = f64.on ? f64.part_b + f64.acoef_b : sep_b;
+    // scratch for `lanes` launch groups at a time.  FP64: where the device has no room for it, the
+    // generic kernels, which need less (none for the single-CTA lengths)
+    auto reserve = [&](int lanes) {
+      const size_t more = lanes > 1 ? 256 : 0;
+      if (f64.on) {
+        const fst_status st = ensure_ws(p, lanes * f64.inter_b + more + f64.part_b + f64.acoef_b);
+        if (st != FST_ENOMEM) return st;
+        f64.on = false;
+      }
+      return ensure_ws(p, lanes * ws_need(Lc, dbl, (int)p->rpad, false) + more + sep_b);
+    };
     auto run = [&]() { return f64.on ? run_f64(p, f64, a, npairs, (char *)p->ws) : run_conv<T>(R, Lc, a, npairs, p->ws); };
     const bool graphs = R->device() && graphs_enabled() && !profiling_enabled() && !tc_stall_pending() &&
                         !R->user_stream_capturing();
     if (!graphs) {
-      TRY(ensure_ws(p, slot + extra));
+      TRY(reserve(1));
       return run();
     }
     // whole apply as one cached CUDA graph (two overlapping lanes of launch groups)
@@ -454,7 +463,7 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
       if (e.y == (const void *)y && e.out == (void *)out && e.batch == batch && e.ld == ld && e.rows_all == a.rows_all &&
           e.dtype == (int)(cplx ? 1 : 0) + (dbl ? 2 : 0) && e.full == full)
         return R->graph_launch(e.exec, e.nodes);
-    TRY(ensure_ws(p, 2 * slot + 256 + extra));
+    TRY(reserve(2));
     if (!R->graph_begin()) return run();
     fst_status st = run();
     const std::string first_err = st != FST_OK ? std::string(g_err) : std::string();

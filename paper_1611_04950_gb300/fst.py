@@ -35,7 +35,7 @@ EXPORTED = ["fst_plan", "fst_plan_op", "fst_plan_info", "fst_plan_export", "fst_
             "fst_launch_count", "fst_profile_enable", "fst_profile_count", "fst_profile_read",
             "fst_project_noalloc", "fst_noalloc_scratch_bytes", "fst_coeffs", "fst_coeffs_info",
             "fst_adi_shifts", "fst_plan_many", "fst_emu_plan_many", "fst_project_ragged", "fst_expand",
-            "fst_sync", "fst_test_tc_stall", "fst_ragged_tuning"]
+            "fst_sync", "fst_test_tc_stall", "fst_test_alloc_fail", "fst_ragged_tuning"]
 
 
 class FSTError(RuntimeError):
@@ -61,6 +61,7 @@ def _load():
         "fst_sync": ([P, vp], I),
         "fst_ragged_tuning": ([C.POINTER(P), C.POINTER(vp), C.POINTER(vp), i64, I, C.POINTER(i64), C.POINTER(d)], I),
         "fst_test_tc_stall": ([I, d], I),
+        "fst_test_alloc_fail": ([I], I),
         "fst_last_error": ([], C.c_char_p),
         "fst_version": ([], C.c_char_p),
         "fst_reduced_tridiagonal": ([i64, d, I, C.POINTER(i64), C.POINTER(d), C.POINTER(d)], I),
@@ -286,6 +287,11 @@ def fst_test_tc_stall(launches: int, limit_s: float = 0.02):
     """Test hook: the next `launches` tensor-core correction launches give up on a wait that
     nothing completes, after limit_s seconds, before issuing any work."""
     _check(_lib.fst_test_tc_stall(launches, limit_s))
+
+
+def fst_test_alloc_fail(allocations: int):
+    """Test hook: the next `allocations` device allocations of the library report a full device."""
+    _check(_lib.fst_test_alloc_fail(allocations))
 
 
 def fst_launch_count() -> int:

@@ -115,3 +115,20 @@ def test_fp64_captured_whatever_ran_before():
         outs.append((out, p))
     assert torch.equal(outs[0][0], outs[1][0])
     assert torch.equal(outs[0][0], outs[0][1].project(y))
+
+
+@pytest.mark.parametrize("graphs", ["1", "0"])
+def test_fp64_short_signals_on_a_full_device(monkeypatch, graphs):
+    # the split kernels' workspace is not to be had: the kernel that needs none answers
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    monkeypatch.setenv("FST_GRAPHS", graphs)
+    p = F.Plan(4096, 1 / 16, eps=1e-6)
+    y = workloads.gaussian(5, 4096, seed=8).to("cuda")
+    F.fst_test_alloc_fail(1)
+    try:
+        got = p.project(y)
+        again = p.project(y, out=torch.empty_like(y))   # with memory again: the split kernels
+    finally:
+        F.fst_test_alloc_fail(0)
+    assert float((got - again).norm()) < 1e-12 * float(y.norm())
