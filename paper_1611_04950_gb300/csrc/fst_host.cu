@@ -208,10 +208,13 @@ static fst_status run_conv(Runner *R, const Layout &L, ConvArgs<T> a, int64_t np
   const bool want = a.mode == MODE_FULL && a.r > 0 && sizeof(T) == 4 && R->device() && !L.small;
   const bool tc = want && tc_usable(*reinterpret_cast<const ConvArgs<float> *>(&a));
   const ConvArgs<float> &af = *reinterpret_cast<const ConvArgs<float> *>(&a);
-  // (at P = 8 and 17 to 64 rows no tensor map can address, the column pass's own products are the
-  // faster ones: 33 rows of 9001 samples 21.1 us, folded 23.6)
+  // (at P = 8 and 17 to 48 rows no tensor map can address, the column pass's own products are the
+  // faster ones.  us, own / folded, N = 9001, r = 26: 17 rows 20.7 / 23.0, 33 rows 22.6 / 25.0,
+  // 48 rows 24.8 / 23.4, 56 rows 29.1 / 27.0; N = 16383, r = 55: 24.8 / 28.9, 27.0 / 28.8,
+  // 31.0 / 32.0, 39.3 / 37.1; r = 5 and N = 8193, 12345 cross at the same place, where the
+  // column pass takes another group of 8 pairs)
   const int64_t nrows = a.rows_all;
-  const bool sym = af.STt && af.cord && !plain_mode() && !(L.fast && L.log2P == 3 && nrows > 16 && nrows <= 64);
+  const bool sym = af.STt && af.cord && !plain_mode() && !(L.fast && L.log2P == 3 && nrows > 16 && nrows <= 48);
   const bool split = want && (L.split_corr || tc || sym);
   ConvArgs<float> sc{};
   if (split) {

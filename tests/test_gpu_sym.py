@@ -59,3 +59,24 @@ def test_tensor_core_correction_rank_33_to_64(N, W, eps, batch, cplx):
     nrm = np.linalg.norm(y.numpy(), axis=1)
     assert np.all(np.linalg.norm(out.cpu().numpy()[pick] - ref, axis=1) < 1e-5 * nrm[pick])
     assert torch.equal(p.project(yd), out)
+
+
+@pytest.mark.parametrize("N", [8193, 16383])
+@pytest.mark.parametrize("batch,cplx", [(48, False), (49, False), (32, True)])
+def test_unaligned_rows_around_the_column_pass_rule(N, batch, cplx):
+    # P = 8, rows no tensor map can address: own products up to 48 rows, folded sums above
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    p = F.Plan(N, 0.2, eps=1e-6)
+    o = O.make_plan(N, 0.2, p.K, 1e-6)
+    y = workloads.gaussian(batch, N, seed=batch, complex_=cplx).to(torch.complex64 if cplx else torch.float32)
+    pick = [0, batch // 2, batch - 1]
+    ref = O.fast_project(o, y.numpy()[pick].astype(np.complex128 if cplx else np.float64).T).T
+    yd = y.to("cuda")
+    F.fst_profile_enable(True)
+    out = p.project(yd)
+    names = {r[0] for r in F.fst_profile_records()}
+    F.fst_profile_enable(False)
+    assert ("k_sym_c" in names) == (batch * (2 if cplx else 1) > 48)
+    nrm = np.linalg.norm(y.numpy(), axis=1)
+    assert np.all(np.linalg.norm(out.cpu().numpy()[pick] - ref, axis=1) < 1e-5 * nrm[pick])
