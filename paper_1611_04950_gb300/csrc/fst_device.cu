@@ -1037,7 +1037,10 @@ struct DevRunner : Runner {
     const int64_t groups = (rows + sy_rows(rows) - 1) / sy_rows(rows), tiles = ((a.N + 1) / 2 + SY_TN - 1) / SY_TN;
     if (groups > 65535 || a.N < 4 * SY_TN) return 0;
     const int64_t most = std::max<int64_t>((a.N + CORR_BLOCK - 1) / CORR_BLOCK, tc_slices(a.N));
-    // ... and more where a thread would otherwise add more than 128 products in a row
+    // ... and more where a thread would otherwise add more than 128 products in a row, as far as those
+    // partials go: up to 64 columns that bound holds, above it the chains reach 16 tiles (192 products at
+    // r = 76, 384 at most).  Error of U2^* y against FP64 there, N = 2^20: r = 72 2.4e-7, r = 91
+    // 2.7e-7 (r = 54, at 128 products, 3.1e-7); on the tensor cores these were 6.0e-7, 6.0e-7 and 3.5e-7.
     const int ntile = sy_tiles(a.ncord, a.r - a.ncord) * (sy_rows(rows) / 8), kg = ntile < 16 ? 16 : 256 / ntile;
     const int64_t want = std::max<int64_t>(3 * (int64_t)sms / groups, (tiles * ((SY_TN / 4 + kg - 1) / kg) * 4 + 127) / 128);
     return (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(tiles, most), want));
