@@ -39,11 +39,11 @@ int fst_plan_is_emulated(fst_plan_t plan);
 fst_status fst_test_tc_stall(int launches, double limit_s);
 
 /*
- * Test hook for calls on a full device: the next `allocations` device allocations of the
- * library (plans, workspaces, ragged batches) fail as cudaMalloc does without memory, and
- * allocate nothing.  0 ends it.  Errors: FST_EINVAL (allocations < 0).
+ * Test hook for calls on a full device: after `after` more device allocations of the
+ * library (plans, workspaces, ragged batches) the next `allocations` ones fail as cudaMalloc
+ * does without memory, and allocate nothing.  (0, 0) ends it.  Errors: FST_EINVAL (negative).
  */
-fst_status fst_test_alloc_fail(int allocations);
+fst_status fst_test_alloc_fail(int after, int allocations);
 
 #ifdef __cplusplus
 }

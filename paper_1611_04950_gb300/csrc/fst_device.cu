@@ -500,13 +500,12 @@ bool tc_stall_take() {
   return false;
 }
 
-// test hook (fst_test_alloc_fail): the next g_alloc_fail device allocations report a full device
-static std::atomic<int> g_alloc_fail{0};
+// test hook (fst_test_alloc_fail): after g_alloc_after more device allocations the next g_alloc_fail
+// ones report a full device
+static std::atomic<int> g_alloc_fail{0}, g_alloc_after{0};
 static bool alloc_fail_take() {
-  int v = g_alloc_fail.load();
-  while (v > 0)
-    if (g_alloc_fail.compare_exchange_weak(v, v - 1)) return true;
-  return false;
+  if (g_alloc_fail.load() <= 0 || g_alloc_after.fetch_sub(1) > 0) return false;
+  return g_alloc_fail.fetch_sub(1) > 0;
 }
 
 static inline int grid_for(int64_t n, int block) {
@@ -1628,6 +1627,7 @@ extern "C" fst_status fst_project_ragged(const fst_plan_t *plans, const void *co
     ctx = new RaggedCtx();
     ctx->sig = sig;
     ctx->plans.assign(plans, plans + count);
+    ctx->state.records = ragged_graphs_enabled();
     g_ragged.push_back(ctx);
   }
   for (int64_t i = 0; i < count; ++i) plans[i]->R->set_stream(stream);
@@ -1704,8 +1704,9 @@ extern "C" fst_status fst_ragged_tuning(const fst_plan_t *plans, const void *con
   return fail(FST_EINVAL, "no ragged call with this signature has run");
 }
 
-extern "C" fst_status fst_test_alloc_fail(int allocations) {
-  if (allocations < 0) return fail(FST_EINVAL, "bad allocation count");
+extern "C" fst_status fst_test_alloc_fail(int after, int allocations) {
+  if (after < 0 || allocations < 0) return fail(FST_EINVAL, "bad allocation count");
+  fst::g_alloc_after.store(after);
   fst::g_alloc_fail.store(allocations);
   return FST_OK;
 }

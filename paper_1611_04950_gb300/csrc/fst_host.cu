@@ -1897,7 +1897,8 @@ static fst_status ragged_fourstep_f32(const fst_plan_t *plans, const void *const
     st.tune_ms.assign(32, 0.0);
   }
   // an intermediate workspace for each of two lanes of classes (256 MiB at most): a class goes to
-  // the lane with less work so far, longest first
+  // the lane with less work so far, longest first.  One lane where no recording makes use of a second,
+  // or the device has no room for it.
   size_t ws_max = 0;
   for (int lg = 0; lg < 32; ++lg)
     if (!cls[lg].empty())
@@ -1905,14 +1906,20 @@ static fst_status ragged_fourstep_f32(const fst_plan_t *plans, const void *const
                                     ((size_t)8 << lg));
   void *dws[2];
   double load[2] = {0.0, 0.0};
-  for (int k = 0; k < 2; ++k) TRY(ragged_buf(R, st, ws_max, nullptr, &dws[k]));
   std::vector<int> order;
   for (int lg = 0; lg < 32; ++lg)
     if (!cls[lg].empty()) order.push_back(lg);
+  if (!st.lanes) st.lanes = st.records && !inplace_any && order.size() > 1 ? 2 : 1;
+  TRY(ragged_buf(R, st, ws_max, nullptr, &dws[0]));
+  if (st.lanes == 2) {
+    const fst_status ws2 = ragged_buf(R, st, ws_max, nullptr, &dws[1]);
+    if (ws2 == FST_ENOMEM) st.lanes = 1;
+    else TRY(ws2);
+  }
   auto work = [&](int lg) { return (double)cls[lg].size() * (double)(1LL << lg); };
   std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return work(p) > work(q); });
   for (int lg : order) {
-    const int lane = load[1] < load[0] ? 1 : 0;
+    const int lane = st.lanes == 2 && load[1] < load[0] ? 1 : 0;
     load[lane] += work(lg);
     if (br && lane) TRY(R->branch(1));
     else TRY(R->branch(-1));

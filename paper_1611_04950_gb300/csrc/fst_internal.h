@@ -253,6 +253,8 @@ bool profiling_enabled();   // per-launch event timing is on (fst_profile_enable
 // call allocates in a fixed order, later calls with the same signature reuse them in that order
 struct RaggedState {
   bool branches = false;            // recording: independent parts of the batch go to branches
+  bool records = true;              // later calls may be recorded
+  int lanes = 0;                    // lanes of length classes with an intermediate of their own (0: not chosen yet)
   std::vector<void *> bufs;
   size_t next = 0;                  // cursor into bufs during a call
   bool tuned = false;

@@ -61,7 +61,7 @@ def _load():
         "fst_sync": ([P, vp], I),
         "fst_ragged_tuning": ([C.POINTER(P), C.POINTER(vp), C.POINTER(vp), i64, I, C.POINTER(i64), C.POINTER(d)], I),
         "fst_test_tc_stall": ([I, d], I),
-        "fst_test_alloc_fail": ([I], I),
+        "fst_test_alloc_fail": ([I, I], I),
         "fst_last_error": ([], C.c_char_p),
         "fst_version": ([], C.c_char_p),
         "fst_reduced_tridiagonal": ([i64, d, I, C.POINTER(i64), C.POINTER(d), C.POINTER(d)], I),
@@ -289,9 +289,10 @@ def fst_test_tc_stall(launches: int, limit_s: float = 0.02):
     _check(_lib.fst_test_tc_stall(launches, limit_s))
 
 
-def fst_test_alloc_fail(allocations: int):
-    """Test hook: the next `allocations` device allocations of the library report a full device."""
-    _check(_lib.fst_test_alloc_fail(allocations))
+def fst_test_alloc_fail(allocations: int, after: int = 0):
+    """Test hook: after `after` more device allocations of the library the next `allocations` ones
+    report a full device."""
+    _check(_lib.fst_test_alloc_fail(after, allocations))
 
 
 def fst_launch_count() -> int:
