@@ -1845,7 +1845,8 @@ static bool autotune_enabled() {
 //   3. out_i += S_T,i a_i over all items (one launch).
 // While a batch is recorded (st.branches) 1. runs on a branch beside 2., whose classes share two
 // lanes, and so do the single-CTA signals; only 3. waits for all of it.  Signals in place keep the
-// order (1. reads what 2. overwrites).  256 signals of 1000 .. 262144 samples: 736 -> 563 us.
+// order (1. reads what 2. overwrites).  256 signals of 1000 .. 262144 samples: 736 -> 545 us (560 with the
+// second lane forked at its first class, after all of the longest one).
 // The pairs per launch group of each class are picked on the first call (autotuner: the
 // candidate groupings of 16 .. 256 MiB of intermediate are timed with device events and the
 // fastest kept; the grouping does not change the arithmetic, so results do not depend on it).
@@ -1915,6 +1916,11 @@ static fst_status ragged_fourstep_f32(const fst_plan_t *plans, const void *const
     const fst_status ws2 = ragged_buf(R, st, ws_max, nullptr, &dws[1]);
     if (ws2 == FST_ENOMEM) st.lanes = 1;
     else TRY(ws2);
+  }
+  // the second lane begins here, beside the first class and not after it
+  if (br && st.lanes == 2) {
+    TRY(R->branch(1));
+    TRY(R->branch(-1));
   }
   auto work = [&](int lg) { return (double)cls[lg].size() * (double)(1LL << lg); };
   std::stable_sort(order.begin(), order.end(), [&](int p, int q) { return work(p) > work(q); });
