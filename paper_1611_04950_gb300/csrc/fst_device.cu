@@ -600,11 +600,6 @@ struct DevRunner : Runner {
 
   int lanes() const override { return capturing ? 2 : 1; }
   void use_lane(int i) override { cur = capturing ? cap[i & 1] : s; }
-  void lanes_after_first() override {
-    if (!capturing) return;
-    cudaEventRecord(ev_mid, cap[0]);
-    cudaStreamWaitEvent(cap[1], ev_mid, 0);
-  }
   void lanes_join_first() override {
     if (!capturing) return;
     cudaEventRecord(ev_mid, cap[1]);

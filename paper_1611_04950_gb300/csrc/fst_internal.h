@@ -35,8 +35,6 @@ struct Runner {
   virtual bool user_stream_capturing() { return false; }
   virtual int lanes() const { return 1; }
   virtual void use_lane(int) {}
-  // order lane 1 after everything lane 0 has issued so far
-  virtual void lanes_after_first() {}
   // order lane 0 after everything lane 1 has issued so far
   virtual void lanes_join_first() {}
   // side lane (capture only): the separate correction runs there, beside the first passes

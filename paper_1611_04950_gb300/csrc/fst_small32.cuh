@@ -10,7 +10,7 @@
 //     row pieces (rpad / 4 threads per row), S_T a sample by sample from the K-major copy of S_T,
 //     whose columns are coalesced along the samples.
 // Bound: FP32 issue and the S_T reads from L2 (both copies of the half, once per pair).
-// Measured, 999 signals of N = 3001, r = 25: 273 -> 65.
+// Measured, 999 signals of N = 3001, r = 25: 273 -> 65 us.
 #pragma once
 #include "fst_fast.cuh"
 
@@ -226,7 +226,7 @@ __device__ __forceinline__ void small32_body(const SmallPlan &p, const float2 *t
     if (j + T * t < N) store(j + T * t, o[t]);
 }
 
-// grid: pairs; T threads; at least 2048 resident threads' worth of registers (64 each)
+// grid: pairs; T threads; 1024 resident threads per SM, whose 64 registers each fill the register file
 template <int LM>
 __global__ void __launch_bounds__((1 << LM) / 16, 1024 / ((1 << LM) / 16)) k_small32(const ConvArgs<float> a,
                                                                                      const SmallPlan p) {
