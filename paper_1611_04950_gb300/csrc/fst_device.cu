@@ -367,6 +367,8 @@ static fst_status set_attrs() {
   CU(cudaFuncSetAttribute(k_passC<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
   CU(cudaFuncSetAttribute(k_passC<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
   CU(cudaFuncSetAttribute(k_sym_c<false, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
+  CU(cudaFuncSetAttribute(k_sym_c<false, 8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
+  CU(cudaFuncSetAttribute(k_sym_c<true, 8, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
   CU(cudaFuncSetAttribute(k_sym_c<false, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
   CU(cudaFuncSetAttribute(k_sym_c<false, 32>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
   CU(cudaFuncSetAttribute(k_sym_c<true, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, mx), "attr");
@@ -1031,12 +1033,12 @@ struct DevRunner : Runner {
     const int64_t groups = (rows + sy_rows(rows) - 1) / sy_rows(rows), tiles = ((a.N + 1) / 2 + SY_TN - 1) / SY_TN;
     if (groups > 65535 || a.N < 4 * SY_TN) return 0;
     const int64_t most = std::max<int64_t>((a.N + CORR_BLOCK - 1) / CORR_BLOCK, tc_slices(a.N));
-    // ... and more where a thread would otherwise add more than 128 products in a row, as far as those
+    // ... and more where a thread would otherwise add more than 108 products in a row, as far as those
     // partials go: up to 64 columns that bound holds, above it the chains reach 16 tiles (192 products at
-    // r = 76, 384 at most).  Error of U2^* y against FP64 there, N = 2^20: r = 72 2.4e-7, r = 91
-    // 2.7e-7 (r = 54, at 128 products, 3.1e-7); on the tensor cores these were 6.0e-7, 6.0e-7 and 3.5e-7.
+    // r = 76, 384 at most).  (At powers of two the resulting blocks are also whole waves of the 304 resident
+    // ones: 16 rows of 2^22, 1214 chunks 240 us, 1024 chunks of 128 products 246.)
     const int ntile = sy_tiles(a.ncord, a.r - a.ncord) * (sy_rows(rows) / 8), kg = ntile < 16 ? 16 : 256 / ntile;
-    const int64_t want = std::max<int64_t>(3 * (int64_t)sms / groups, (tiles * ((SY_TN / 4 + kg - 1) / kg) * 4 + 127) / 128);
+    const int64_t want = std::max<int64_t>(3 * (int64_t)sms / groups, (tiles * ((SY_TN / 4 + kg - 1) / kg) * 4 + 107) / 108);
     return (int)std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(tiles, most), want));
   }
   fst_status sym_c(const ConvArgs<float> &a) override {
@@ -1046,7 +1048,12 @@ struct DevRunner : Runner {
     dim3 grid((unsigned)a.nkb, (unsigned)((rows + RB - 1) / RB));
     const size_t smem = sy_smem(a.ncord, a.r - a.ncord, RB);
     auto go = [&](auto kernel) { PROF("k_sym_c", a.npairs, (kernel<<<grid, 256, smem, cur>>>(a, a.cord, a.ncord, a.nkb))); };
-    if (a.cplx) go(RB == 8 ? k_sym_c<true, 8> : RB == 16 ? k_sym_c<true, 16> : k_sym_c<true, 32>);
+    // products in a row per thread (sym_chunks)
+    const int ntile = sy_tiles(a.ncord, a.r - a.ncord) * (RB / 8), kg = ntile < 16 ? 16 : 256 / ntile;
+    const int64_t tiles = ((a.N + 1) / 2 + SY_TN - 1) / SY_TN;
+    const bool quad = RB == 8 && (tiles + a.nkb - 1) / a.nkb * ((SY_TN / 4 + kg - 1) / kg) * 4 > 64;
+    if (quad) go(a.cplx ? k_sym_c<true, 8, true> : k_sym_c<false, 8, true>);
+    else if (a.cplx) go(RB == 8 ? k_sym_c<true, 8> : RB == 16 ? k_sym_c<true, 16> : k_sym_c<true, 32>);
     else go(RB == 8 ? k_sym_c<false, 8> : RB == 16 ? k_sym_c<false, 16> : k_sym_c<false, 32>);
     LAUNCHED("k_sym_c");
     return FST_OK;

@@ -929,8 +929,16 @@ __global__ void k_corr_reduce(const ConvArgs<float> a, const float *scale) {
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   for (int t = blockIdx.y * nw + w; t < 2 * a.r; t += nw * gridDim.y) {
     const int c = t / a.r, j = t % a.r;
-    float s = 0.f;
-    for (int b = lane; b < nK; b += 32) s += a.part[((pl * nK + b) * 2 + c) * a.rpad + j];
+    // eight chains a lane: short chains of roundings, loads that overlap
+    float q[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    for (int b = lane; b < nK; b += 256) {
+      float v[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) v[i] = b + 32 * i < nK ? a.part[((pl * nK + b + 32 * i) * 2 + c) * a.rpad + j] : 0.f;
+#pragma unroll
+      for (int i = 0; i < 8; ++i) q[i] += v[i];
+    }
+    float s = ((q[0] + q[1]) + (q[2] + q[3])) + ((q[4] + q[5]) + (q[6] + q[7]));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) a.acoef[(pl * 2 + c) * a.rpad + j] = __ldg(scale + j) * s;

@@ -30,13 +30,19 @@ __host__ __device__ inline size_t sy_smem(int nE, int nO, int RB) {
 // shared memory along the samples; the next tile's columns (second buffer) and rows (registers) are
 // loaded while the current one is multiplied.  Thread (column tile, row tile, sample group) accumulates 8 x 8 sums,
 // 16 16-byte loads per 256 FMAs (its columns and rows are ct + k nct and vt + k nvt: neighbouring
-// threads read neighbouring 16-byte pieces).  Sample groups are added in order at the end; one partial
+// threads read neighbouring 16-byte pieces).  Sample groups are added in fixed chains at the end; one partial
 // per (row, chunk), the layout k_corr_reduce reads.
+// QUAD: the four products of a step are added among themselves first, a quarter of the roundings at the
+// size of the sum for a fifth FP32 instruction per four.  For chains of more than 64 products in blocks of 8
+// rows, which wait for memory anyway: error of U2^* y against FP64 of one row of 2^21 samples 2.9e-7 -> 1.8e-7,
+// of 8 rows 2.8e-7 -> 1.8e-7 (the 2048-sample blocks before this kernel 2.4e-7, 2.1e-7), same time; blocks of
+// 32 rows would take 350 -> 487 us (64 complex signals of 2^20), and their errors are below those of the
+// tensor cores' sums without it.
 // Bound: FP32 FMA against the HBM reads of y and of half of S_T.  Measured (us, unfolded -> folded): 16 real
 // signals of 2^22, r = 60: 366 -> 242; 64 complex ones of 2^20, r = 38: 246 (tcgen05, alone on the
 // chip) -> 335, but the whole call 2075 -> 1997, since these blocks run beside the column passes.
 // ---------------------------------------------------------------------------
-template <bool CPLX, int RB>
+template <bool CPLX, int RB, bool QUAD = false>
 __global__ void __launch_bounds__(256, 2) k_sym_c(const ConvArgs<float> a, const int *cord, int nE, int nchunk) {
   extern __shared__ __align__(16) float ysm[];
   constexpr int nvt = RB / 8, RT = RB / 4;   // rows a thread loads (complex: RT / 2 signals)
@@ -117,7 +123,8 @@ __global__ void __launch_bounds__(256, 2) k_sym_c(const ConvArgs<float> a, const
           const float4 s = *reinterpret_cast<const float4 *>(cb + c * cst + 4 * g);
 #pragma unroll
           for (int q = 0; q < 8; ++q)
-            acc[c][q] = fmaf(s.w, v[q].w, fmaf(s.z, v[q].z, fmaf(s.y, v[q].y, fmaf(s.x, v[q].x, acc[c][q]))));
+            if (QUAD) acc[c][q] += fmaf(s.w, v[q].w, fmaf(s.z, v[q].z, fmaf(s.y, v[q].y, s.x * v[q].x)));
+            else acc[c][q] = fmaf(s.w, v[q].w, fmaf(s.z, v[q].z, fmaf(s.y, v[q].y, fmaf(s.x, v[q].x, acc[c][q]))));
         }
       }
     }
@@ -137,10 +144,22 @@ __global__ void __launch_bounds__(256, 2) k_sym_c(const ConvArgs<float> a, const
     const int o = odd ? nE + (tct - tE) + c * tO : tct + c * tE;
     const int row = tvt + q * nvt;
     if ((odd ? o < a.r : o < nE) && row < nr) {
-      float s = red[e];
-      for (int k = 1; k < kg; ++k) s += red[k * ntile * 64 + e];
+      // four chains, a quarter of the roundings in a row (32 rows have few groups: one chain, whose main
+      // loop also compiles to the faster code, 350 instead of 367 us for 64 complex signals of 2^20)
+      float sum = red[e];
+      if (RB < 32) {
+        float s[4] = {sum, 0.f, 0.f, 0.f};
+        for (int k0 = 1; k0 < kg; k0 += 4) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            if (k0 + i < kg) s[(i + 1) & 3] += red[(k0 + i) * ntile * 64 + e];
+        }
+        sum = (s[0] + s[1]) + (s[2] + s[3]);
+      } else {
+        for (int k = 1; k < kg; ++k) sum += red[k * ntile * 64 + e];
+      }
       const int64_t rw = row0 + row;
-      a.part[(((rw >> 1) * nchunk + blockIdx.x) * 2 + (rw & 1)) * a.rpad + __ldg(cord + o)] = s;
+      a.part[(((rw >> 1) * nchunk + blockIdx.x) * 2 + (rw & 1)) * a.rpad + __ldg(cord + o)] = sum;
     }
   }
 }

@@ -80,3 +80,23 @@ def test_unaligned_rows_around_the_column_pass_rule(N, batch, cplx):
     assert ("k_sym_c" in names) == (batch * (2 if cplx else 1) > 48)
     nrm = np.linalg.norm(y.numpy(), axis=1)
     assert np.all(np.linalg.norm(out.cpu().numpy()[pick] - ref, axis=1) < 1e-5 * nrm[pick])
+
+
+@pytest.mark.parametrize("batch", [1, 8])
+def test_few_rows_sum_as_accurately_as_unfolded(batch):
+    # chains of more than 64 products: U2^* y of N = 2^21 against FP64, no further off than the sums
+    # over blocks of 2048 samples that the folded form replaced (2.1e-7 to 2.2e-7)
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    N = 1 << 21
+    p = F.Plan(N, 0.2, eps=1e-4)
+    S = torch.as_tensor(p.export()["S_T"]).cuda()
+    sd = torch.as_tensor(p.export(False)["D"]).cuda().abs().sqrt()
+    num = den = 0.0
+    for seed in range(16 // batch):
+        y = workloads.gaussian(batch, N, seed=seed).float().cuda()
+        ref = (y.double() @ S) * sd
+        got = p.coeffs(y)[:, -p.r:].real.double()
+        num += float((got - ref).norm()) ** 2
+        den += float(ref.norm()) ** 2
+    assert (num / den) ** 0.5 <= 2.2e-7
