@@ -575,18 +575,25 @@ static Reduced reduced_tridiagonal(int64_t N, double W, int parity) {
   return R;
 }
 
+// exp(-2 pi i k / 2^24), 0 <= k < 2^24, from the angle to the nearest multiple of pi/2: an angle near
+// 2 pi in double is off by up to 4.4e-16 before its cosine is taken, four times the rounding of the
+// result (FP64 projections of N = 100003 were 6.0e-16 off with it, 3.8e-16 without)
+static double2 unit_root(int k) {
+  const int quarter = 1 << (TW_LOG2 - 2), q = (k + quarter / 2) / quarter;
+  const double x = 2.0 * M_PI * ((double)(k - q * quarter) / (double)(1 << TW_LOG2));   // |x| <= pi / 4
+  const double c = cos(x), s = sin(x);
+  switch (q & 3) {
+    case 0: return make_double2(c, -s);
+    case 1: return make_double2(-s, -c);
+    case 2: return make_double2(-c, s);
+    default: return make_double2(s, c);
+  }
+}
 static void build_twiddles(std::vector<double2> &hi, std::vector<double2> &lo) {
   hi.resize(TW_HI_SIZE);
   lo.resize(TW_LO_SIZE);
-  // exp(-2 pi i k / 2^24); the angle fraction k / 2^24 is exact in double
-  for (int a = 0; a < TW_HI_SIZE; ++a) {
-    const double f = (double)((int64_t)a << TW_SPLIT) / (double)(1 << TW_LOG2);
-    hi[a] = make_double2(cos(2.0 * M_PI * f), -sin(2.0 * M_PI * f));
-  }
-  for (int b = 0; b < TW_LO_SIZE; ++b) {
-    const double f = (double)b / (double)(1 << TW_LOG2);
-    lo[b] = make_double2(cos(2.0 * M_PI * f), -sin(2.0 * M_PI * f));
-  }
+  for (int a = 0; a < TW_HI_SIZE; ++a) hi[a] = unit_root(a << TW_SPLIT);
+  for (int b = 0; b < TW_LO_SIZE; ++b) lo[b] = unit_root(b);
 }
 
 static double asymptotic_transition(int64_t N, double eps) {

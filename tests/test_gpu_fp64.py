@@ -132,3 +132,28 @@ def test_fp64_short_signals_on_a_full_device(monkeypatch, graphs):
     finally:
         F.fst_test_alloc_fail(0)
     assert float((got - again).norm()) < 1e-12 * float(y.norm())
+
+
+@pytest.mark.parametrize("N,W", [(4096, 1 / 16), (100003, 0.1)])
+def test_fp64_rounding_against_long_double(N, W):
+    # B y of a pair by FFTs in long double (64 or more bits of mantissa).  Kernels that form their twiddles as
+    # products of a few small angles' roots are off by 3.8e-16 and 5.1e-16 here; a table entry per
+    # factor has one rounding instead of up to three, so it may not be further off
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    fft = pytest.importorskip("scipy.fft")
+    L = np.longdouble
+    if np.finfo(L).eps > 1e-18 or fft.rfft(np.ones(4, L)).dtype != np.clongdouble:
+        pytest.skip("no extended precision")
+    pi = L("3.14159265358979323846264338327950288")
+    k = np.arange(1, N).astype(L)
+    x = 2 * L(W) * k
+    b = np.concatenate([[2 * L(W)], np.sin(pi * (x - 2 * np.floor(x / 2))) / (pi * k)])
+    M = 1 << (2 * N - 1).bit_length()
+    c = np.concatenate([b, np.zeros(M - 2 * N + 1, L), b[:0:-1]])
+    y = workloads.gaussian(2, N, seed=N)
+    B = fft.rfft(c)
+    ref = np.stack([fft.irfft(B * fft.rfft(np.concatenate([v.astype(L), np.zeros(M - N, L)])), n=M)[:N] for v in y.numpy()])
+    got = F.Plan(N, W, eps=1e-6).apply_prolate(y.cuda()).cpu().numpy()
+    err = np.sqrt(((got - ref) ** 2).sum() / (ref ** 2).sum())
+    assert err < (3.8e-16 if N == 4096 else 5.1e-16), err
