@@ -15,7 +15,7 @@
 //     is symmetric or antisymmetric, s_l(N-1-n) = (-1)^l s_l(n), so the FMAs of S_T^T y and of
 //     S_T a halve.
 // Measured (us, before -> after): one pair of N = 4096 479 -> 40; 64 signals of N = 40000,
-// r = 32, 1977 -> 1283.
+// r = 32, 1977 -> 1275.
 #pragma once
 #include "fst_kernels.cuh"
 
