@@ -439,7 +439,7 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
     // which needs none.  Longer ones need a workspace with any kernels and make do with what is there,
     // so that the same call records the same arithmetic whatever the plan has run before (a batch whose
     // coefficients alone fill it: the generic kernels).
-    const bool recording = dbl && R->user_stream_capturing();
+    const bool recording = R->user_stream_capturing();
     F64Plan f64;
     if (dbl && !(recording && p->lay64.small))
       f64 = f64_plan(p, *reinterpret_cast<const ConvArgs<double> *>(&a), npairs, full, recording ? std::max<size_t>(1, p->ws_bytes) : 0);
@@ -455,8 +455,7 @@ static fst_status apply_t(fst_plan_t p, const T *y, T *out, int64_t batch, int64
       return ensure_ws(p, lanes * ws_need(Lc, dbl, (int)p->rpad, false) + more + sep_b);
     };
     auto run = [&]() { return f64.on ? run_f64(p, f64, a, npairs, (char *)p->ws) : run_conv<T>(R, Lc, a, npairs, p->ws); };
-    const bool graphs = R->device() && graphs_enabled() && !profiling_enabled() && !tc_stall_pending() &&
-                        !R->user_stream_capturing();
+    const bool graphs = R->device() && graphs_enabled() && !profiling_enabled() && !tc_stall_pending() && !recording;
     if (!graphs) {
       TRY(reserve(1));
       return run();
