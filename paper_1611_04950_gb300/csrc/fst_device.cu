@@ -1200,18 +1200,34 @@ struct DevRunner : Runner {
     LAUNCHED("k_coef_gemm");
     return FST_OK;
   }
-  static int exp_spt(int64_t nsig) { return nsig >= 32 ? 4 : (nsig >= 16 ? 2 : 1); }
+  // vectors a thread: one, from 16 vectors two, from 32 four, but only as many as leave two blocks for
+  // every SM, in number and in shared memory (more of them share the columns' loads, fewer spread the
+  // batch).  us at N = 4096, eps = 1e-6, one / two / four: 64 vectors 35.0 / 34.9 / 41.1, 128 47.2 / 41.1 /
+  // 43.1, 256 69.8 / 59.5 / 54.8; N = 128, 64 vectors 24.7 / 27.1 / 32.9; N = 32768, eps = 1e-10 (four: one
+  // block per SM), 64 vectors 116 / 101 / 119
+  int exp_spt(int64_t N, int rH, int DA, int DB, int r, int64_t nsig) const {
+    const int64_t tiles = N / 2 / LR_TN;
+    int spt = nsig >= 32 ? 4 : (nsig >= 16 ? 2 : 1);
+    while (spt > 1 && (tiles * ((nsig + 4 * spt - 1) / (4 * spt)) <= 2 * sms ||
+                       2 * exp_smem(rH, DA, DB, r, spt) > 226 * 1024))
+      spt /= 2;
+    return spt;
+  }
   static size_t exp_smem(int rH, int DA, int DB, int r, int spt) {
     return (size_t)8 * spt * xp_words(rH, DA, DB, r) * 8 + (size_t)LR_TN * xp_cs(rH, DA, DB, r) * 4;
   }
   size_t expand_scratch(int64_t N, int rH, int DA, int DB, int r, int64_t nsig) override {
+    // few short vectors with few columns: the generic kernel, one launch less (us, generic / shared columns:
+    // N = 128, rH = 7, 64 vectors 20.6 / 22.6; N = 256, rH = 8, 16 20.6 / 22.6; N = 1024, rH = 7, 64 24.7 / 26.7;
+    // but N = 256, rH = 8, 256 vectors 24.7 / 22.6; N = 1024, rH = 9, 64 28.8 / 26.7)
+    if (N <= 1024 && rH <= 8 && nsig * rH <= 1024) return 0;
     if (N < 2 * LR_TN || exp_smem(rH, DA, DB, r, 4) > 227 * 1024) return 0;
     return (size_t)nsig * xp_words(rH, DA, DB, r) * 8 + 256;
   }
   fst_status expand_gemm(const ExpArgs<float> &a, int64_t nsig, void *scratch, const unsigned char *cpar) override {
     TRY(set_attrs());
     float2 *cc = (float2 *)scratch;
-    const int nw = xp_words(a.rH, a.DA, a.DB, a.r), spt = exp_spt(nsig);
+    const int nw = xp_words(a.rH, a.DA, a.DB, a.r), spt = exp_spt(a.N, a.rH, a.DA, a.DB, a.r, nsig);
     PROF("k_exp_prep", nsig, (k_exp_prep<<<grid_for(nsig * nw, 256), 256, 0, cur>>>(a, nsig, cc)));
     LAUNCHED("k_exp_prep");
     // vectors split until there are about four blocks per SM, in whole rounds of 8 spt vectors

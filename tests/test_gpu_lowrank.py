@@ -33,3 +33,25 @@ def test_lowrank_against_fp64(N, W, eps, batch, cplx):
     x = p.expand(got)
     want = p.expand(got.to(torch.complex128))
     assert bool(((x.to(torch.complex128) - want).norm(dim=1) <= 2e-6 * want.norm(dim=1)).all())
+
+
+@pytest.mark.parametrize("N,W,eps,batch,shared", [(128, 0.1, 1e-8, 3, True), (128, 0.2, 1e-6, 40, True), (128, 0.2, 1e-3, 146, False),
+                                                  (128, 0.2, 1e-3, 147, True), (256, 0.1, 1e-8, 700, True),
+                                                  (1024, 0.2, 1e-2, 64, False), (2048, 0.1, 1e-10, 50, True),
+                                                  (4096, 0.2, 1e-6, 130, True), (4096, 0.2, 1e-6, 260, True)])
+def test_expand_route_and_vectors_per_thread(N, W, eps, batch, shared):
+    # the generic kernel for few short vectors with few columns; one, two and four vectors a thread
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    p = F.Plan(N, W, eps=eps)
+    rH = F.fst_coeffs_info(p.h)["rH"]
+    assert shared == (not (N <= 1024 and rH <= 8 and batch * rH <= 1024))
+    y = workloads.gaussian(batch, N, seed=4, complex_=True).to("cuda")
+    c = p.coeffs(y.to(torch.complex64))
+    F.fst_profile_enable(True)
+    x = p.expand(c)
+    names = {r[0] for r in F.fst_profile_records()}
+    F.fst_profile_enable(False)
+    assert ("k_expand_gemm" in names) == shared
+    want = p.expand(c.to(torch.complex128))
+    assert bool(((x.to(torch.complex128) - want).norm(dim=1) <= 2e-6 * want.norm(dim=1)).all())
