@@ -125,7 +125,8 @@ fst_status fst_plan_export(fst_plan_t plan, int64_t *idx, double *lam, double *D
  * 16-byte aligned, its row stride is a multiple of 16 bytes and the batch has more than
  * 32 signal rows (real signals, or two per complex signal), S_T^T y for the whole batch
  * runs on the tensor cores (TF32 with a hi/lo split, three products); other batches use
- * FP32 CUDA-core sums over the folded half of S_T -- other summation orders, same
+ * FP32 CUDA-core sums over the folded half of S_T, or for some of at most 48 rows
+ * three-product TF32 sums inside the first FFT pass -- other summation orders, same
  * accuracy.  The number of partial sums follows the batch in FP64 (N > 256) and in the
  * folded form.  Results are bit-for-bit repeatable for the same call.
  * Workspace: kept by the plan and grown on demand, at most two launch groups of 128 MiB

@@ -208,13 +208,17 @@ static fst_status run_conv(Runner *R, const Layout &L, ConvArgs<T> a, int64_t np
   const bool want = a.mode == MODE_FULL && a.r > 0 && sizeof(T) == 4 && R->device() && !L.small;
   const bool tc = want && tc_usable(*reinterpret_cast<const ConvArgs<float> *>(&a));
   const ConvArgs<float> &af = *reinterpret_cast<const ConvArgs<float> *>(&a);
-  // (at P = 8 and 17 to 48 rows no tensor map can address, the column pass's own products are the
-  // faster ones.  us, own / folded, N = 9001, r = 26: 17 rows 20.7 / 23.0, 33 rows 22.6 / 25.0,
-  // 48 rows 24.8 / 23.4, 56 rows 29.1 / 27.0; N = 16383, r = 55: 24.8 / 28.9, 27.0 / 28.8,
-  // 31.0 / 32.0, 39.3 / 37.1; r = 5 and N = 8193, 12345 cross at the same place, where the
-  // column pass takes another group of 8 pairs)
+  // (rows no tensor map can address: the column pass's own products are the faster ones at P = 8 from 17 to
+  // 48 rows and at P = 16, and P = 32 with few columns, from 33 to 48; at 48 it takes another group of 8
+  // pairs.  us, own / folded:
+  // N = 8193, r = 28: 16 rows 18.6 / 18.4, 17 18.6 / 22.5, 33 20.6 / 27.9, 48 24.7 / 22.8, 56 28.8 / 25.4;
+  // N = 12345, r = 44: 22.6 / 20.7, 22.7 / 26.7, 24.7 / 28.7, 28.8 / 32.5, 35.0 / 34.6;
+  // N = 30001, r = 48: 24 rows 33.9 / 31.9, 33 39.0 / 40.7, 48 41.1 / 45.0, 56 56.6 / 51.5;
+  // P = 32: N = 65535, r = 18: 32 rows 43.2 / 42.7, 33 47.9 / 53.3, 48 55.5 / 58.0, 56 78.8 / 70.9;
+  // N = 40001, r = 32: 33 53.3 / 49.6; N = 50001, r = 50: 33 71.7 / 65.6, 48 79.3 / 73.9)
   const int64_t nrows = a.rows_all;
-  const bool sym = af.STt && af.cord && !plain_mode() && !(L.fast && L.log2P == 3 && nrows > 16 && nrows <= 48);
+  const bool own = L.fast && (L.log2P <= 4 || a.rpad <= 24) && nrows > (L.log2P == 3 ? 16 : 32) && nrows <= 48;
+  const bool sym = af.STt && af.cord && !plain_mode() && !own;
   const bool split = want && (L.split_corr || tc || sym);
   ConvArgs<float> sc{};
   if (split) {

@@ -100,3 +100,25 @@ def test_few_rows_sum_as_accurately_as_unfolded(batch):
         num += float((got - ref).norm()) ** 2
         den += float(ref.norm()) ** 2
     assert (num / den) ** 0.5 <= 2.2e-7
+
+
+@pytest.mark.parametrize("N,eps,batch,own", [(8193, 1e-6, 16, False), (8193, 1e-6, 17, True), (20001, 1e-6, 32, False),
+                                             (20001, 1e-6, 33, True), (32767, 1e-6, 48, True), (30001, 1e-6, 49, False),
+                                             (40001, 1e-6, 40, False), (40001, 1e-3, 40, True)])
+def test_unaligned_rows_by_column_count(N, eps, batch, own):
+    # which of P = 8, 16, 32 keeps the column pass's own products, and that both forms agree with the oracle
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    p = F.Plan(N, 0.2, eps=eps)
+    o = O.make_plan(N, 0.2, p.K, eps)
+    y = workloads.gaussian(batch, N, seed=batch).float()
+    pick = [0, batch // 2, batch - 1]
+    ref = O.fast_project(o, y.numpy()[pick].astype(np.float64).T).T
+    yd = y.to("cuda")
+    F.fst_profile_enable(True)
+    out = p.project(yd)
+    names = {r[0] for r in F.fst_profile_records()}
+    F.fst_profile_enable(False)
+    assert ("k_sym_c" not in names) == own
+    nrm = np.linalg.norm(y.numpy(), axis=1)
+    assert np.all(np.linalg.norm(out.cpu().numpy()[pick] - ref, axis=1) < 1e-5 * nrm[pick])
